@@ -186,6 +186,35 @@ __device__ __forceinline__ float cell_lower_bound2(const Grid& g, float qx, floa
     return s * (1.0f - 0x1p-20f);
 }
 
+// The rows of the box [lx, lx + ex) x [ly, ly + ey) x [lz, lz + ez) through
+// the row index, one row per lane and 32 per step: each is one range of pts,
+// cut to the chord of the smaller of tau and the current k-th distance.  A
+// box of half-width R cells costs ~(2R + 1) row lookups per level of z where
+// the hash costs (2R + 1)^2 cell probes, so the search can widen to any
+// distance; the per-row cut drops the rows that the k found so far exclude.
+// Measured (131k-point scan searched with itself, k = 20; the 700 to 1,000
+// queries in its sparse rim find their 20th neighbour up to 100 cells away
+// and, cell by cell, ended in the scan of every occupied cell): 9.8-36 ms
+// by cells, 0.73-0.89 ms by rows; k = 48, 20k queries of a 300k map, where
+// every query takes this search: 0.209 -> 0.188 ms.
+template <int SLOTS>
+__device__ void scan_rows(const Grid& g, float qx, float qy, float qz, int lx, int ly, int lz,
+                          int ex, int ey, int ez, float eta, float tau, SearchState<SLOTS>& S, u64* pend,
+                          int k, int lane, uint32_t ibase) {
+    const int64_t nrows = (int64_t)ey * ez;
+    for (int64_t base = 0; base < nrows; base += 32) {
+        const int64_t r = base + lane;
+        uint2 v = make_uint2(0u, 0u);
+        if (r < nrows) {
+            const int cz = lz + (int)(r / ey), cy = ly + (int)(r % ey);
+            const float kd = S.kth == EMPTY_KEY ? INFINITY : __uint_as_float((uint32_t)(S.kth >> 32));
+            const float tm = fminf(tau, kd);
+            v = row_part(g, qx, qy, qz, cy, cz, lx, lx + ex - 1, eta, tm, tm * (1.0f + 0x1p-18f));
+        }
+        scan_ranges(g, qx, qy, qz, v.x, v.y, tau, S, pend, k, lane, ibase);
+    }
+}
+
 template <int SLOTS>
 __device__ void scan_box(const Grid& g, float qx, float qy, float qz, int lx, int ly, int lz,
                          int ex, int ey, int ez, float tau, SearchState<SLOTS>& S, u64* pend,
@@ -238,7 +267,8 @@ struct WarpBox {
     int lx, ly, lz;
     int ex, ey, ez;
     int64_t ncl;
-    float tau;
+    float tau, eta;
+    bool all;  // the box holds the whole window range: nothing is left outside it
 };
 
 __device__ __forceinline__ WarpBox warp_box(const Grid& g, float qx, float qy, float qz, float rho) {
@@ -257,7 +287,31 @@ __device__ __forceinline__ WarpBox warp_box(const Grid& g, float qx, float qy, f
     b.ey = max(min(hy, g.why) - b.ly + 1, 0);
     b.ez = max(min(hz, g.whz) - b.lz + 1, 0);
     b.ncl = (int64_t)b.ex * b.ey * b.ez;
+    const int cm = max(max(max(abs(lx), abs(hx + 1)), max(abs(ly), abs(hy + 1))), max(abs(lz), abs(hz + 1)));
+    const float qm = fmaxf(fabsf(qx), fmaxf(fabsf(qy), fabsf(qz)));
+    b.eta = 0x1p-20f * (g.coord_scale + qm + (float)cm * g.h);
+    b.all = lx <= g.wlx && hx >= g.whx && ly <= g.wly && hy >= g.why && lz <= g.wlz && hz >= g.whz;
     return b;
+}
+
+// Whether the widening search may scan this box.  Through the row index (and
+// where the exact scan of every occupied cell is allowed to follow) the cost
+// is its rows: up to as many as there are occupied cells, beyond which that
+// scan is the cheaper one.  Otherwise its cells, up to max_box_cells.
+__device__ __forceinline__ bool box_allowed(const Grid& g, const WarpBox& b) {
+    if (g.dstart && g.exhaustive)
+        return (int64_t)b.ey * b.ez <= max(g.ncells, (int64_t)4096) || b.ncl <= (int64_t)g.max_box_cells;
+    return b.ncl <= (int64_t)g.max_box_cells;
+}
+
+template <int SLOTS>
+__device__ __forceinline__ void scan_warp_box(const Grid& g, float qx, float qy, float qz, const WarpBox& b, float tau,
+                                              SearchState<SLOTS>& S, u64* pend, int k, int lane, uint32_t ibase) {
+    if (b.ncl <= 0) return;
+    if (g.dstart)
+        scan_rows(g, qx, qy, qz, b.lx, b.ly, b.lz, b.ex, b.ey, b.ez, b.eta, tau, S, pend, k, lane, ibase);
+    else
+        scan_box(g, qx, qy, qz, b.lx, b.ly, b.lz, b.ex, b.ey, b.ez, tau, S, pend, k, lane, ibase);
 }
 
 // Exact k nearest neighbours of one query (warp-uniform control flow).
@@ -276,18 +330,21 @@ __device__ int knn_search(const Grid& g, const Grid& dg, float qx, float qy, flo
         const WarpBox b = warp_box(g, qx, qy, qz, rho);
         WarpBox d = b;
         float tau = b.tau;
+        bool all = b.all;
         if (DEL) {
             d = warp_box(dg, qx, qy, qz, rho);
             tau = fminf(tau, d.tau);
-            if (d.ncl > (int64_t)dg.max_box_cells) break;
+            all = all && d.all;
+            if (!box_allowed(dg, d)) break;
         }
-        if (b.ncl > (int64_t)g.max_box_cells) break;
+        if (!box_allowed(g, b)) break;
+        if (all && g.exhaustive) tau = INFINITY;  // no point lies outside the box
         state_reset(S);
-        if (b.ncl > 0) scan_box(g, qx, qy, qz, b.lx, b.ly, b.lz, b.ex, b.ey, b.ez, tau, S, pend, k, lane, 0u);
-        if (DEL && d.ncl > 0)
-            scan_box(dg, qx, qy, qz, d.lx, d.ly, d.lz, d.ex, d.ey, d.ez, tau, S, pend, k, lane, (uint32_t)g.m);
+        scan_warp_box(g, qx, qy, qz, b, tau, S, pend, k, lane, 0u);
+        if (DEL) scan_warp_box(dg, qx, qy, qz, d, tau, S, pend, k, lane, (uint32_t)g.m);
         flush(S, pend, k, lane);
         if (S.kth != EMPTY_KEY) return SEARCH_OK;
+        if (all && g.exhaustive) return SEARCH_SHORT;  // every point of the window was seen
         int found = 0;
 #pragma unroll
         for (int s = 0; s < SLOTS; ++s) found += __popc(__ballot_sync(FULL, S.L[s] != EMPTY_KEY));
