@@ -8,58 +8,26 @@
 // tau, so any radius t with t^2 <= tau that holds >= k points holds the k
 // nearest.  Two searches use it:
 //
-// * Lane path (k <= 32; lane_tile) -- one query per lane of a 32-query
-//   tile.  Pass 1 walks the rows of the box (occupancy bitmap + rank, one
-//   contiguous point range per row) and counts points under eight trial
-//   radii; the smallest radius holding >= k (and <= the survivor cap)
-//   wins, a failing lane retries with the radii scaled, and pass 2
-//   collects the winners' positions in shared memory.  A register odd-even
-//   merge sort network sorts 32-bit keys (d2 bits with a slot tag), an exact fix-up
-//   orders equal buckets by (d2, index), and the covariance reads the k
-//   neighbours from the cell-sorted copy in rank order.
-// * Warp path (k > 32, and the lane path's leftovers; knn_search) -- one
-//   query per warp: the cells of a radius-driven box are looked up in the
-//   voxel hash one per lane, candidates arrive 32 at a time as coalesced
-//   float4 loads, survivors of the certified filter are merged into a
-//   register top-k by bitonic shuffles, and the radius widens until k are
-//   certified; past max_box_cells an exact scan over all occupied cells
-//   (or PC_ERR_SEARCH_LIMIT) ends it.
+// * Group search (k <= 32; group_unit): four or eight lanes per query walk
+//   the rows of the box (one contiguous point range per row), keep the points
+//   within the radius in shared memory, and sort the survivors by (d2, index).
+// * Warp path (k > 32, and in knn_rest.cu the group search's leftovers;
+//   knn_search): one query per warp, the rows of a widening box read one per
+//   lane (cells through the hash where there is no row index), candidates 32
+//   at a time, survivors merged into a register top-k by bitonic shuffles.
 //
 // The covariance is a two-pass binary32 mean/centred sum shifted by the
-// nearest neighbour; for eps >= 0 a binary32 Jacobi eigen-solve gives the
-// normal n and C' = I - (1-eps) n n^T.  Nothing here changes a result bit
+// nearest neighbour; for eps >= 0 a closed-form binary32 eigen-solve gives
+// the normal n and C' = I - (1-eps) n n^T.  Nothing here changes a result bit
 // with the tile, launch shape, radii, tile order or batching.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <mutex>
 
 #include "knn_kernels.cuh"
 
 // ---------------------------------------------------------------- host side
 namespace {
-
-// Opt every search kernel (both window variants) into large dynamic shared
-// memory, once per device (outside any stream capture: the first launch or
-// plan does it).
-std::mutex g_attr_mu;
-unsigned g_attr_done = 0u;
-cudaError_t ensure_attrs() {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const unsigned bit = 1u << (dev & 31);
-    std::lock_guard<std::mutex> lk(g_attr_mu);
-    if (g_attr_done & bit) return cudaSuccess;
-    if ((e = allow_all_smem<false>()) != cudaSuccess) return e;
-    if ((e = pc_knn_win_attrs()) != cudaSuccess) return e;
-    if ((e = pc_knn_union_attrs()) != cudaSuccess) return e;
-    if ((e = pc_knn_union_win_attrs()) != cudaSuccess) return e;
-    g_attr_done |= bit;
-    return cudaSuccess;
-}
-
-int clamp_tile(int t) { return t <= 0 ? 32 : (t > 32 ? 32 : t); }
 
 // The search mode for k on this target: its tune may ask for 64 survivor
 // slots (mode 1) for every k <= 32.
@@ -69,67 +37,63 @@ int target_mode(const pc_target_s* t, int k) {
 }
 int clamp_warps(int w) { return w <= 0 ? 4 : (w > 8 ? 8 : w); }
 
-// Calls f(kernel) with the search kernel for (mode, with_cov, windowed).
-template <bool BATCH, typename F>
-cudaError_t with_kernel(int mode, bool with_cov, bool windowed, F&& f, bool stage = false) {
-    void* kern = windowed ? pc_knn_kernel_win(mode, with_cov, BATCH, stage)
-                          : knn_kernel<false>(mode, with_cov, BATCH, stage);
-    return f(kern);
+// Lanes per query of the group search.  Eight shorten a query's chain of
+// dependent loads where a call cannot fill the chip; four do less work.
+// Measured, us with 4 / 8 lanes at 6k, 20k, 48k queries: track map, k = 20
+// 29 / 22, 32 / 29, 40 / 48; k = 10 27 / 21, 27 / 24, 34 / 37; k = 32 41 / 27,
+// 42 / 33, 51 / 55; uniform box, k = 20 46 / 34, 53 / 50, 78 / 80.
+int group_lanes(int64_t n) { return n <= 24576 ? 8 : 4; }
+
+// Launches the search kernel of (form, mode, covariance kind, window) over
+// its work items: one per one-warp block of the group search, one per warp of
+// the warp path.
+cudaError_t launch_form(int form, const Grid& g, int mode, int cov, int64_t tiles, int tile, int warps, void** args,
+                        cudaStream_t s) {
+    if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+    const int group = mode < 2 ? 32 / tile : 1;
+    void* kern = g.windowed ? pc_knn_kernel_win(form, mode, cov, group)
+               : form == 2  ? pc_knn_kernel_union(mode, cov, group)
+               : form == 1  ? pc_knn_kernel_batch(mode, cov, group)
+                            : knn_kernel<0, false>(mode, cov, group);
+    if (mode < 2) warps = 1;
+    return cudaLaunchKernel(kern, dim3((unsigned)((tiles + warps - 1) / warps)), dim3(32 * warps), args, 0, s);
+}
+
+int cov_kind(bool with_cov, const CovKernel& ck) { return !with_cov ? 0 : (ck.type == 0 ? 1 : 2); }
+
+TileArgs tile_args(const pc_target_s* t, const CovKernel& ck, int k, float eps, bool host_cov) {
+    return TileArgs{k, eps, t->tune.order == 0 ? 1 : 0, ck, host_cov ? 1 : 0, pc_probe_c(t)};
 }
 
 }  // namespace
 
+int pc_search_tile(const pc_target_s* t, int k, int64_t n) {
+    if (target_mode(t, k) < 2) return 32 / group_lanes(n);
+    return t->tune.tile <= 0 ? 32 : std::min(t->tune.tile, 32);
+}
+
+// The covariance (plain, or weighted by the target's kernel descriptor) is
+// fused into the search.  With appended points the main grid and the delta
+// grid are searched as one map.
 cudaError_t pc_launch_knn(const pc_target_s* t, const float* q, int64_t N, int k, float eps,
-                          int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s, bool stage) {
+                          int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s,
+                          bool host_cov) {
     if (N == 0) return cudaSuccess;
-    cudaError_t e = ensure_attrs();
-    if (e != cudaSuccess) return e;
-    const int tile = clamp_tile(t->tune.tile);
-    const int warps = clamp_warps(t->tune.warps);
-    // the covariance (plain, or weighted by the target's kernel descriptor)
-    // is fused into the search
-    const bool with_cov = cov != nullptr;
-    const int mode = target_mode(t, k);
-    stage = stage && mode < 2 && with_cov;  // the warp path writes its rows directly
-    TileArgs a{k, eps, t->tune.rho_scale > 0 ? t->tune.rho_scale : 0.9f, t->tune.order == 0 ? 1 : 0, t->ck,
-               pc_probe_c(t)};
-    const size_t smem = (size_t)warps * warp_bytes(mode, stage, k);
+    const int tile = pc_search_tile(t, k, N), mode = target_mode(t, k), warps = clamp_warps(t->tune.warps);
     const int64_t tiles = (N + tile - 1) / tile;
-    const int64_t blocks = (tiles + warps - 1) / warps;
-    Grid g = t->g;
-    float* covp = with_cov ? cov : nullptr;
-    void* args[] = {&g, (void*)&q, (void*)&N, (void*)&tile, &a, &rho0, &idx, &d2, &covp};
-    return with_kernel<false>(
-        mode, with_cov, g.windowed != 0,
-        [&](void* kern) { return cudaLaunchKernel(kern, dim3((unsigned)blocks), dim3(warps * 32), args, smem, s); },
-        stage);
+    TileArgs a = tile_args(t, t->ck, k, eps, host_cov);
+    Grid g = t->g, dg = t->delta ? t->delta->g : t->g;
+    cudaError_t e;
+    if (t->delta) {
+        void* args[] = {&g, &dg, (void*)&q, (void*)&N, (void*)&tile, &a, &rho0, &idx, &d2, &cov};
+        e = launch_form(2, g, mode, cov_kind(cov != nullptr, t->ck), tiles, tile, warps, args, s);
+    } else {
+        void* args[] = {&g, (void*)&q, (void*)&N, (void*)&tile, &a, &rho0, &idx, &d2, &cov};
+        e = launch_form(0, g, mode, cov_kind(cov != nullptr, t->ck), tiles, tile, warps, args, s);
+    }
+    if (e != cudaSuccess || mode == 2) return e;
+    return pc_launch_rest(g, t->delta ? &dg : nullptr, q, N, tile, a, rho0, idx, d2, cov, s);
 }
-
-// The union search (a target with appended points): the same launch shape
-// as pc_launch_knn over the main grid and the delta grid together.
-cudaError_t pc_launch_knn_union(const pc_target_s* t, const float* q, int64_t N, int k, float eps,
-                                int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s) {
-    if (N == 0) return cudaSuccess;
-    cudaError_t e = ensure_attrs();
-    if (e != cudaSuccess) return e;
-    const int tile = clamp_tile(t->tune.tile);
-    const int warps = clamp_warps(t->tune.warps);
-    const bool with_cov = cov != nullptr;
-    const int mode = target_mode(t, k);
-    TileArgs a{k, eps, t->tune.rho_scale > 0 ? t->tune.rho_scale : 0.9f, t->tune.order == 0 ? 1 : 0, t->ck,
-               pc_probe_c(t)};
-    const size_t smem = (size_t)warps * warp_smem_bytes(mode);
-    const int64_t tiles = (N + tile - 1) / tile;
-    const int64_t blocks = (tiles + warps - 1) / warps;
-    Grid g = t->g;
-    Grid dg = t->delta->g;
-    float* covp = with_cov ? cov : nullptr;
-    void* args[] = {&g, &dg, (void*)&q, (void*)&N, (void*)&tile, &a, &rho0, &idx, &d2, &covp};
-    void* kern = g.windowed ? pc_knn_union_kernel_win(mode, with_cov) : pc_knn_union_kernel(mode, with_cov);
-    return cudaLaunchKernel(kern, dim3((unsigned)blocks), dim3(warps * 32), args, smem, s);
-}
-
-cudaError_t pc_knn_prepare() { return ensure_attrs(); }
 
 cudaError_t pc_launch_cov(const pc_target_s* t, const int32_t* idx, int64_t N, int k, float eps,
                           float* cov, cudaStream_t s) {
@@ -141,23 +105,15 @@ cudaError_t pc_launch_cov(const pc_target_s* t, const int32_t* idx, int64_t N, i
 }
 
 cudaError_t pc_launch_knn_batch(const pc_target_s* t, const Grid& gv, const CovKernel& ck,
-                                const ScanDesc* scans_dev, int nscans, int64_t max_n,
-                                int64_t total_tiles, int tile, int warps, int k, float eps,
-                                bool with_cov, float rho0, cudaStream_t s, bool stage) {
+                                const ScanDesc* scans_dev, int nscans, int64_t total_tiles, int64_t queries,
+                                int tile, int warps, int k, float eps, bool with_cov, bool host_cov, float rho0,
+                                cudaStream_t s) {
     if (total_tiles == 0) return cudaSuccess;
-    cudaError_t e = ensure_attrs();
-    if (e != cudaSuccess) return e;
-    TileArgs a{k, eps, t->tune.rho_scale > 0 ? t->tune.rho_scale : 0.9f, t->tune.order == 0 ? 1 : 0, ck,
-               pc_probe_c(t)};
-    const int64_t blocks = (total_tiles + warps - 1) / warps;
-    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
     const int mode = target_mode(t, k);
-    stage = stage && mode < 2;  // the warp path writes its rows directly
-    const size_t smem = (size_t)warps * warp_bytes(mode, stage, k);
+    TileArgs a = tile_args(t, ck, k, eps, host_cov);
     Grid g = gv;
     void* args[] = {&g, (void*)&scans_dev, &nscans, &total_tiles, &tile, &a, &rho0};
-    return with_kernel<true>(
-        mode, with_cov, g.windowed != 0,
-        [&](void* kern) { return cudaLaunchKernel(kern, dim3((unsigned)blocks), dim3(warps * 32), args, smem, s); },
-        stage);
+    const cudaError_t e = launch_form(1, g, mode, cov_kind(with_cov, ck), total_tiles, tile, warps, args, s);
+    if (e != cudaSuccess || mode == 2) return e;
+    return pc_launch_rest_batch(g, scans_dev, nscans, total_tiles, queries, tile, a, rho0, s);
 }

@@ -497,6 +497,20 @@ __device__ __forceinline__ void cov_finish(float cxx, float cxy, float cxz, floa
            1.0f - f * n.z * n.z);
 }
 
+// C' = I - (1 - eps) n n^T in place of a packed covariance; eps < 0 keeps the
+// covariance.
+__device__ __forceinline__ void cov_regularise(float* c, float eps) {
+    if (eps < 0.0f) return;
+    const float3 n = min_eigvec(c[0], c[1], c[2], c[3], c[4], c[5]);
+    const float f = 1.0f - eps;
+    c[0] = 1.0f - f * n.x * n.x;
+    c[1] = -f * n.x * n.y;
+    c[2] = -f * n.x * n.z;
+    c[3] = 1.0f - f * n.y * n.y;
+    c[4] = -f * n.y * n.z;
+    c[5] = 1.0f - f * n.z * n.z;
+}
+
 template <typename G>
 __device__ __forceinline__ void cov_core(G&& get, int k, float eps, float* out) {
     const float4 p0 = get(0);
@@ -672,14 +686,6 @@ __device__ void weighted_core(G&& get, const CovKernel& ck, float qx, float qy, 
 }
 
 // ---------------------------------------------------------------- tiles
-struct TileArgs {
-    int k;
-    float eps;
-    float rho_scale;
-    int last_first;  // issue tiles from the end of the query array
-    CovKernel ck;    // kernel-descriptor weights; type 0: the plain covariance
-    float probe_c;   // > 0: each lane estimates its own starting radius (probe_radius)
-};
 
 // The covariance of a written row (caller or union indices; a leading -1
 // marks an unanswered row), plain or weighted by the descriptor in a.
@@ -700,35 +706,57 @@ __device__ void cov_row_any(const Grid& g, const Grid& dg, const int32_t* nb, in
     }, a.ck, qx, qy, qz, k, a.eps, out);
 }
 
-// Per-warp shared memory: 64 staged survivor keys of the warp-cooperative
-// search, then the lane path's survivor lists: 32 slots x 32 lanes of
-// positions into pts ([slot][lane], so a slot is one 128-byte row).
-// Search modes: 0 = lane path with room for 32 survivors (k <= 24),
-// 1 = lane path with room for 64 (k <= 32), 2 = warp path only (k > 32).
-__host__ __device__ __forceinline__ int lane_cap(int mode) { return mode == 0 ? 32 : mode == 1 ? 64 : 0; }
-__host__ __device__ __forceinline__ int search_mode(int k) { return k <= 24 ? 0 : (k <= 32 ? 1 : 2); }
-__host__ __device__ __forceinline__ size_t warp_smem_bytes(int mode) {
-    return 64 * sizeof(u64) + (size_t)lane_cap(mode) * 32 * sizeof(uint32_t);
-}
-// Staging area of a warp whose outputs go to host memory: the tile's idx
-// rows, d2 rows and covariance rows, each laid out as in the output arrays.
-__host__ __device__ __forceinline__ size_t stage_bytes(int k) { return (size_t)32 * (2 * k + 6) * sizeof(float); }
-__host__ __device__ __forceinline__ size_t warp_bytes(int mode, bool stage, int k) {
-    return warp_smem_bytes(mode) + (stage ? stage_bytes(k) : 0);
-}
+// ---------------------------------------------------------------- group search
+// k <= 32: a group of G lanes (4, or 8 for small calls) answers a query, and a
+// block is one warp: a unit of 32 / G queries.
+//
+// 1. Walk: the rows of the box around the starting radius are resolved one
+//    per lane and handed round the group, whose lanes take the points of G
+//    rows in turn as one run.  Every point with d2 <= t = min(r^2, tau), tau
+//    certified for the box, goes to the lane's list in shared memory (d2 and
+//    position).  With at least k points and no list overflowing, the k
+//    smallest of them are the k nearest overall: all points with d2 <= t lie
+//    in the box.  Otherwise the radius is scaled by what the count says about
+//    the density and the query walks again (131k scan: 1.04 walks a warp).
+// 2. Selection, when the lists hold more than CAP points: thresholds placed
+//    by linear interpolation in d2 (a surface's count grows evenly in d2)
+//    are counted over the lists, four at a time, until one holds between k
+//    and CAP points.
+// 3. Sort: 32-bit keys (d2 bits << 1, low TB bits replaced by the list slot)
+//    sorted across the group: Batcher's network on each lane's CAP / G
+//    registers, then bitonic merges between lanes.  The keys order d2 to
+//    within 2^(TB-1) ulps; a group that finds two neighbours in one such
+//    bucket is put in exact (d2, index) order by an insertion sort.
+// 4. Rows are written by the warp as one contiguous block; three lanes of
+//    the group carry the covariance sums.
+//
+// k_knn_rest follows every launch.  It turns the covariances into normals and
+// C' (eps >= 0), one query per lane, and answers the queries that no attempt
+// settled (fewer than k points within reach, or more than CAP equal
+// distances): their row's first d2 word is UNANSWERED, and the sign bit of
+// the unit's first d2 word marks the unit.  Squared distances are never
+// negative and never NaN, so neither mark can be mistaken for a result, and
+// no workspace or counter is shared between calls in flight.
+//
+// What bounds it: issue slots (68-72 % of them used) in the row walk, two
+// thirds of the time.  One lane per query on blocks of four warps (the layout
+// before) kept 32 different point streams in a warp, walked twice, held 95
+// registers and ran 1.35 waves of long warps.
+constexpr int MAX_ATTEMPTS = 6;
+constexpr float START = 1.4f;  // first radius over the calibrated starting radius; 1.26 and 1.54: 8 and 12 % slower
+constexpr int BATCH = 2;       // point loads a lane has in flight; 1 and 3: 3 % slower on scans
+constexpr uint32_t UNANSWERED = 0xffffffffu, UNIT_FLAG = 0x80000000u;
+constexpr uint32_t NAN_ROW = 0x7fc00000u;  // every entry of a covariance row without a value
 
-// Copies n words from shared memory to global (or host-mapped) memory with
-// the whole warp: 16-byte vectors when both ends allow it, so each store
-// instruction writes 512 contiguous bytes.
-__device__ __forceinline__ void warp_copy_out(uint32_t* __restrict__ dst, const uint32_t* src, int n, int lane) {
-    int done = 0;
-    if (((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0) {
-        const int n4 = n >> 2;
-        for (int i = lane; i < n4; i += 32)
-            reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
-        done = n4 << 2;
-    }
-    for (int i = done + lane; i < n; i += 32) dst[i] = src[i];
+// Search modes: 0 = group search with room for 32 sorted survivors (k <= 24),
+// 1 = with room for 64 (k <= 32), 2 = warp path only (k > 32).
+__host__ __device__ __forceinline__ int search_mode(int k) { return k <= 24 ? 0 : (k <= 32 ? 1 : 2); }
+// List slots of a lane: 64 (k <= 24) or 96 points per query over G lanes.
+__host__ __device__ constexpr int lane_slots(int cap, int g) { return (cap == 32 ? 64 : 96) / g; }
+// Shared memory of one warp: the lists (d2, position), then CAP sort keys per
+// query.
+__host__ __device__ constexpr size_t group_warp_smem(int cap, int g) {
+    return (size_t)lane_slots(cap, g) * 32 * 8 + (size_t)(32 / g) * cap * sizeof(uint32_t);
 }
 
 __device__ __forceinline__ void cas32(uint32_t& a, uint32_t& b) {
@@ -737,15 +765,11 @@ __device__ __forceinline__ void cas32(uint32_t& a, uint32_t& b) {
     b = hi;
 }
 
-// Batcher's odd-even merge sort over the first NN registers, ascending:
-// merges sorted runs of length p into runs of 2p; within a merge, elements
-// k apart are compared, k halving from p, and only pairs inside the same
-// run of 2p.  The comparator list is computed at compile time and expanded
-// as a parameter pack, so every register index is a constant (NN = 32: 191
-// comparators, where a bitonic network takes 240).  For NN not a power of
-// two the list is the next power of two's less every comparator that
-// reaches past NN: with the registers from NN on holding the largest key,
-// such a comparator never moves anything, so what remains sorts NN keys.
+// Batcher's odd-even merge sort over NN registers, ascending: merges sorted
+// runs of length p into runs of 2p; within a merge, elements k apart are
+// compared, k halving from p, and only pairs inside the same run of 2p.  The
+// comparator list is computed at compile time and expanded as a parameter
+// pack, so every register index is a constant.
 template <int NN>
 struct OemNet {
     struct Table {
@@ -768,399 +792,546 @@ struct OemNet {
     }
 };
 
-template <int NN, int CAP, int... Cs>
-__device__ __forceinline__ void oem_apply(uint32_t (&K)[CAP], std::integer_sequence<int, Cs...>) {
+template <int NN, int... Cs>
+__device__ __forceinline__ void oem_apply(uint32_t (&K)[NN], std::integer_sequence<int, Cs...>) {
     (cas32(K[std::integral_constant<int, OemNet<NN>::make().a[Cs]>::value],
            K[std::integral_constant<int, OemNet<NN>::make().b[Cs]>::value]),
      ...);
 }
 
-template <int NN, int CAP>
-__device__ __forceinline__ void sort_regs(uint32_t (&K)[CAP]) {
+template <int NN>
+__device__ __forceinline__ void sort_regs(uint32_t (&K)[NN]) {
     oem_apply<NN>(K, std::make_integer_sequence<int, OemNet<NN>::make().n>{});
 }
 
-// Trial radii of the lane path, as multiples of the starting radius: a
-// geometric ladder from 0.75 to 1.46.  With 32 survivor slots (k <= 24) the
-// ladder has eight steps of ratio 1.1, so the count at the chosen radius is
-// at most ~1.2x the smallest count that reaches k on a surface and seldom
-// overflows the slots; with 64 slots four steps of ratio ~1.22 leave room
-// for the ~1.5x overshoot, and counting four radii instead of eight makes
-// the first pass cheaper (k = 32: 0.148 -> 0.132 ms on the C2 scan).
-template <int CAP>
-struct Ladder {
-    static constexpr int N = CAP == 32 ? 8 : 4;
-    __device__ static __forceinline__ float mul(int j) {
-        if (CAP == 32)
-            return j == 0 ? 0.75f : j == 1 ? 0.83f : j == 2 ? 0.91f : j == 3 ? 1.0f
-                 : j == 4 ? 1.1f : j == 5 ? 1.21f : j == 6 ? 1.33f : 1.46f;
-        return j == 0 ? 0.8f : j == 1 ? 1.0f : j == 2 ? 1.22f : 1.46f;
-    }
-};
-
-// (d2, index) key of the survivor in a lane's slot, recomputed from pts.
-template <bool DEL>
-__device__ __forceinline__ u64 slot_key(const Grid& g, const Grid& dg, const uint32_t* posl, int slot,
-                                        int lane, float qx, float qy, float qz) {
-    const uint32_t tp = posl[slot * 32 + lane];
-    const float4 p = pt_at<DEL>(g, dg, tp);
-    const float d = sqdist_pinned(qx, qy, qz, p.x, p.y, p.z);
-    return ((u64)__float_as_uint(d) << 32) | (u64)union_index<DEL>(g, tp, p);
+// Ascending order of a bitonic sequence in NN registers.
+template <int NN>
+__device__ __forceinline__ void merge_regs(uint32_t (&K)[NN]) {
+#pragma unroll
+    for (int s = NN / 2; s >= 1; s >>= 1)
+#pragma unroll
+        for (int i = 0; i < NN; ++i)
+            if ((i & s) == 0) cas32(K[i], K[i + s]);
 }
 
-// A lane's own starting radius where the map's density is uneven: the
+// Sorts the group's G * NN keys: lane sub of the group ends with the keys
+// of ranks sub * NN .. sub * NN + NN - 1.  Runs of w lanes are merged into
+// runs of 2w by comparing each key with its mirror in the other run, which
+// leaves two bitonic halves, then by exchanges between lanes w / 2 .. 1 apart
+// and a merge inside each lane.
+template <int NN, int G>
+__device__ __forceinline__ void sort_group(uint32_t (&K)[NN], int sub) {
+    sort_regs<NN>(K);
+#pragma unroll
+    for (int w = 1; w < G; w <<= 1) {
+        const bool lower = (sub & w) == 0;
+        uint32_t y[NN];
+#pragma unroll
+        for (int i = 0; i < NN; ++i) y[i] = __shfl_xor_sync(FULL, K[NN - 1 - i], 2 * w - 1);
+#pragma unroll
+        for (int i = 0; i < NN; ++i) K[i] = lower ? min(K[i], y[i]) : max(K[i], y[i]);
+#pragma unroll
+        for (int s = w >> 1; s >= 1; s >>= 1) {
+            const bool low = (sub & s) == 0;
+#pragma unroll
+            for (int i = 0; i < NN; ++i) {
+                const uint32_t z = __shfl_xor_sync(FULL, K[i], s);
+                K[i] = low ? min(K[i], z) : max(K[i], z);
+            }
+        }
+        merge_regs<NN>(K);
+    }
+}
+
+// Sum of v over the lanes of a group.
+template <int G>
+__device__ __forceinline__ uint32_t group_sum(uint32_t v) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
+}
+
+// Visits every point of the box [l, h] (clamped to the grid) whose row -- or,
+// without the row index, whose cell -- can hold a point within sqrt(t) of q,
+// as f(position, point), the points of a row spread over the group's lanes.
+// Control flow is uniform over the warp but for the innermost loops; groups
+// with act = false take part with empty boxes.
+template <int G, bool WIN, typename F>
+__device__ __forceinline__ void group_walk(const Grid& g, bool act, float qx, float qy, float qz, int lx, int hx,
+                                           int ly, int hy, int lz, int hz, float eta, float t, int sub,
+                                           uint32_t& visits, F&& f) {
+    const bool rows = g.dstart != nullptr;
+    const int nx = rows ? 1 : hx - lx + 1, ny = hy - ly + 1, nz = hz - lz + 1;
+    const int units = act && lx <= hx && ny > 0 && nz > 0 ? nx * ny * nz : 0;
+    const int last = __reduce_max_sync(FULL, (unsigned)units);
+    const float tx = t * (1.0f + 0x1p-18f);
+    const bool wx = WIN && g.windowed && (lx == g.tlx || hx == g.thx);
+    int cx = lx, cy = ly, cz = lz;
+    auto advance = [&](int n) {
+        if (!rows) {
+            cx += n;
+            n = 0;
+            while (cx > hx) {
+                cx -= nx;
+                ++n;
+            }
+        }
+        cy += n;
+        while (cy > hy) {
+            cy -= ny;
+            ++cz;
+        }
+    };
+    if (sub < units) advance(sub);
+    for (int base = 0; base < last; base += G) {
+        uint2 r = make_uint2(0u, 0u);
+        if (base + sub < units) {
+            if (rows) {
+                r = row_part(g, qx, qy, qz, cy, cz, lx, hx, eta, t, tx);
+            } else {
+                const float lb2 = box_gap2(g, qx, qy, qz, cx, cy, cz, eta);
+                if (!(lb2 * (1.0f - 0x1p-20f) > t)) r = lookup_cell(g, pack_key(cx, cy, cz, g.bx, g.by));
+            }
+            visits += r.y;
+            // a row (cell) on a boundary cell of the window tests its points
+            if (WIN && g.windowed &&
+                ((rows ? wx : cx == g.tlx || cx == g.thx) || cy == g.tly || cy == g.thy || cz == g.tlz ||
+                 cz == g.thz))
+                r.y |= 0x80000000u;
+            advance(G);
+        }
+        // The G rows as one run of c points: point i of it is pts[i + off],
+        // off set by the last row that starts at or before i.
+        uint32_t start[G], upto[G];  // of row j: start less the points before it; points before row j + 1
+        uint32_t c = 0, test = 0;
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            const uint32_t cj = __shfl_sync(FULL, r.y, j, G);
+            start[j] = __shfl_sync(FULL, r.x, j, G) - c;
+            if (WIN) test |= (cj >> 31) << j;
+            c += WIN ? cj & 0x7fffffffu : cj;
+            upto[j] = c;
+        }
+        for (uint32_t i0 = sub; i0 < c; i0 += G * BATCH) {
+            float4 p[BATCH];
+            uint32_t pos[BATCH];
+#pragma unroll
+            for (int b = 0; b < BATCH; ++b) {
+                const uint32_t i = i0 + G * b;
+                uint32_t off = start[0];
+                bool cut = WIN && (test & 1u);
+#pragma unroll
+                for (int j = 1; j < G; ++j)
+                    if (i >= upto[j - 1]) {
+                        off = start[j];
+                        if (WIN) cut = test >> j & 1u;
+                    }
+                pos[b] = i + off;
+                if (i < c) p[b] = window_cut<WIN>(g, cut, __ldg(&g.pts[pos[b]]));
+            }
+#pragma unroll
+            for (int b = 0; b < BATCH; ++b)
+                if (i0 + G * b < c) f(pos[b], p[b]);
+        }
+    }
+}
+
+// The starting radius of a query where the map's density is uneven: the
 // points of the 27 cells around q (counted through the row index, no point
 // is read) set a surface density n / (9 h^2), and the radius of a disc
-// holding k points at that density, c h sqrt(k / n), is where the trial
-// radii start; at most 3 h (and 3 h when the block is empty).  Only the
-// search's speed depends on it.
-template <bool WIN>
-__device__ __forceinline__ float probe_radius(const Grid& g, float qx, float qy, float qz, int k, float c) {
-    const int cx = cell_of(qx, g.ox, g.inv_h), cy = cell_of(qy, g.oy, g.inv_h), cz = cell_of(qz, g.oz, g.inv_h);
-    const int x0 = max(cx - 1, WIN ? g.wlx : 0), x1 = min(cx + 1, WIN ? g.whx : g.dimx - 1);
-    const int y0 = max(cy - 1, WIN ? g.wly : 0), y1 = min(cy + 1, WIN ? g.why : g.dimy - 1);
-    const int z0 = max(cz - 1, WIN ? g.wlz : 0), z1 = min(cz + 1, WIN ? g.whz : g.dimz - 1);
+// holding k points at that density is c h sqrt(k / n); at most 3 h (and 3 h
+// when the block is empty).  Only the search's speed depends on it.
+template <int G, bool WIN>
+__device__ __forceinline__ float probe_radius(const Grid& g, bool act, float qx, float qy, float qz, int k, float c,
+                                              int sub) {
     uint32_t n = 0;
-    if (g.dstart && x0 <= x1)
-        for (int z = z0; z <= z1; ++z)
-            for (int y = y0; y <= y1; ++y) n += row_range(g, y, z, x0, x1).y;
+    if (act && g.dstart) {
+        const int cx = cell_of(qx, g.ox, g.inv_h), cy = cell_of(qy, g.oy, g.inv_h), cz = cell_of(qz, g.oz, g.inv_h);
+        const int x0 = max(cx - 1, WIN ? g.wlx : 0), x1 = min(cx + 1, WIN ? g.whx : g.dimx - 1);
+        const int y0 = max(cy - 1, WIN ? g.wly : 0), y1 = min(cy + 1, WIN ? g.why : g.dimy - 1);
+        const int z0 = max(cz - 1, WIN ? g.wlz : 0), z1 = min(cz + 1, WIN ? g.whz : g.dimz - 1);
+        const int ny = y1 - y0 + 1, nz = z1 - z0 + 1;
+        if (x0 <= x1 && ny > 0 && nz > 0)
+            for (int u = sub; u < ny * nz; u += G) n += row_range(g, y0 + u % ny, z0 + u / ny, x0, x1).y;
+    }
+    n = group_sum<G>(n);
     const float cap = 3.0f * g.h;
     return n > 0 ? fminf(c * g.h * sqrtf((float)k / (float)n), cap) : cap;
 }
 
-// k <= 32: one query per lane.  Pass 1 counts, for each trial radius
-// r_j = m_j rho0, the target points with d2 <= t_j = min(r_j^2, tau), tau
-// certified for the box around the largest radius; the smallest t_j that
-// holds >= k points (and at most CAP) is exact by the same argument as the
-// warp search: every point with d2 <= t_j lies in the box, so the k
-// smallest of those are the k smallest overall.  Pass 2 collects their
-// positions in the lane's shared-memory list.  They are ordered by a
-// register odd-even merge sort network on 32-bit keys (d2 bits << 1, low five
-// bits replaced by the slot), which orders d2 to within 16 ulps; any run of
-// neighbours left in the same 16-ulp bucket is then put in exact (d2,
-// index) order by bubble passes on the full keys.  Lanes whose query needs
-// a wider radius, more than 32 survivors or a bigger box are finished by
-// the warp-cooperative search, one query at a time.
-//
-// With DEL the search covers the union of the main grid g and the grid dg of
-// appended points (point j of dg is g.m + j): both grids' boxes of the trial
-// radius are counted and collected in the same passes, filtered by the
-// smaller of their certified taus, and list entries from dg carry DTAG.
-//
-// With STG the outputs are page-locked host memory: each lane writes its
-// idx/d2 row and covariance into the warp's staging area `stg` (laid out as
-// the output arrays), and the warp copies each array's block of the tile out
-// in 16-byte vectors, so host memory receives whole lines instead of the
-// lanes' scattered 16-byte pieces.
-template <int CAP, bool COV, bool WIN, bool DEL, bool STG>
-__device__ void lane_tile(const Grid& g, const Grid& dg, const float* __restrict__ q, int64_t n0, int cnt,
-                          const TileArgs& a, float rho0, int32_t* __restrict__ idx,
-                          float* __restrict__ d2, float* __restrict__ cov, u64* pend,
-                          uint32_t* posl, uint32_t* stg, int lane) {
-    constexpr int NRAD = Ladder<CAP>::N;
-    auto rad_mul = [](int jj) { return Ladder<CAP>::mul(jj); };
-    const int k = a.k;
-    const bool active = lane < cnt;
-    const int64_t n = n0 + lane;
-    // With STG the rows go to the warp's staging area (laid out as in the
-    // output arrays) and are copied out as one block per tile.
-    int32_t* const si = reinterpret_cast<int32_t*>(stg);
-    float* const sd = reinterpret_cast<float*>(stg + 32 * k);
-    float* const sc = reinterpret_cast<float*>(stg + 64 * k);
-    float qx = 0.0f, qy = 0.0f, qz = 0.0f;
-    if (active) {
-        qx = __ldg(q + 3 * n);
-        qy = __ldg(q + 3 * n + 1);
-        qz = __ldg(q + 3 * n + 2);
+// The cell box of half-width r around q on one grid, clamped to the grid (or
+// its window range), with its certified tau and eta; big: too many rows or
+// cells for a group (k_knn_rest takes those).
+struct GroupBox {
+    int lx, hx, ly, hy, lz, hz;
+    float tau, eta;
+    bool big;
+};
+template <bool WIN>
+__device__ __forceinline__ GroupBox group_box(const Grid& g, float qx, float qy, float qz, float r) {
+    const int lx = cell_of(__fsub_rn(qx, r), g.ox, g.inv_h), hx = cell_of(__fadd_rn(qx, r), g.ox, g.inv_h);
+    const int ly = cell_of(__fsub_rn(qy, r), g.oy, g.inv_h), hy = cell_of(__fadd_rn(qy, r), g.oy, g.inv_h);
+    const int lz = cell_of(__fsub_rn(qz, r), g.oz, g.inv_h), hz = cell_of(__fadd_rn(qz, r), g.oz, g.inv_h);
+    GroupBox b;
+    b.tau = certified_tau(g, qx, qy, qz, lx, hx, ly, hy, lz, hz);
+    const int cm = max(max(max(abs(lx), abs(hx + 1)), max(abs(ly), abs(hy + 1))), max(abs(lz), abs(hz + 1)));
+    const float qm = fmaxf(fabsf(qx), fmaxf(fabsf(qy), fabsf(qz)));
+    b.eta = 0x1p-20f * (g.coord_scale + qm + (float)cm * g.h);
+    b.lx = max(lx, WIN ? g.wlx : 0);
+    b.hx = min(hx, WIN ? g.whx : g.dimx - 1);
+    b.ly = max(ly, WIN ? g.wly : 0);
+    b.hy = min(hy, WIN ? g.why : g.dimy - 1);
+    b.lz = max(lz, WIN ? g.wlz : 0);
+    b.hz = min(hz, WIN ? g.whz : g.dimz - 1);
+    const int64_t nrows = (int64_t)max(b.hy - b.ly + 1, 0) * max(b.hz - b.lz + 1, 0);
+    const int64_t ncl = nrows * max(b.hx - b.lx + 1, 0);
+    b.big = ncl > 4096 || nrows > 256 || (!g.dstart && ncl > 256);
+    return b;
+}
+
+// The covariance of a query from its k neighbours' coordinates in rank order
+// (c[r CS], c[(KMAX + r) CS], c[(2 KMAX + r) CS] for x, y, z of rank r; the
+// next KMAX CS entries are free for weights).  Lane sub < 3 of the group
+// carries one coordinate u: its mean, its square sum and its product sum with
+// the next coordinate v, divided into uu and uv.  Every sum runs over the
+// ranks in order with the operations of cov_core / weighted_core, so the
+// results are theirs bit for bit: the split is over the sums, not over the
+// neighbours.  Returns the divisor (k, or the total weight).
+template <int CS, int KMAX, int G, bool weighted>
+__device__ __forceinline__ float group_moments(float* c, const TileArgs& a, float qx, float qy, float qz, int sub,
+                                               float& uu, float& uv) {
+    const int k = a.k, cu = sub < 3 ? sub : 0, cv = cu == 2 ? 0 : cu + 1;
+    const float* u = c + cu * KMAX * CS;
+    const float* v = c + cv * KMAX * CS;
+    float* const wt = c + 3 * KMAX * CS;
+    const float u0 = u[0], v0 = v[0];
+    float total = (float)k, s = 0.0f;
+    uu = uv = 0.0f;
+    if constexpr (weighted) {
+        for (int j = sub; j < k; j += G)
+            wt[j * CS] = kd_weight(a.ck, qx, qy, qz,
+                                   make_float4(c[j * CS], c[(KMAX + j) * CS], c[(2 * KMAX + j) * CS], 0.0f));
+        __syncwarp();
+        total = 0.0f;
+        for (int j = 0; j < k; ++j) {
+            const float w = wt[j * CS];
+            total = total + w;
+            s = __fmaf_rn(w, u[j * CS] - u0, s);
+        }
+    } else {
+#pragma unroll 4
+        for (int j = 0; j < k; ++j) s = s + (u[j * CS] - u0);
     }
-    const bool finite = active && isfinite(qx) && isfinite(qy) && isfinite(qz);
-    bool fallback = false;
-    int m = 0;
-    float thr = -1.0f;
-    uint32_t visits = 0;  // candidate points whose distance this lane computed
-    int lx = 0, hx = -1, ly = 0, hy = -1, lz = 0, hz = -1;
-    float eta = 0.0f;
-    int dlx = 0, dhx = -1, dly = 0, dhy = -1, dlz = 0, dhz = -1;
-    float deta = 0.0f;
-    // Up to three lane-parallel attempts: a lane whose largest trial radius
-    // held fewer than k points retries with the radii x1.8.  A lane whose
-    // count jumped from below k at one radius to above CAP at the next (a
-    // wall entering the ball between two rungs) retries with thresholds
-    // spaced evenly in d2 between those two radii, where a surface's count
-    // grows evenly; one whose smallest radius held more than CAP retries
-    // with the radii x0.7.  Only lanes that still fail go to the warp
-    // search, whose latency (tens of microseconds for one query) would
-    // otherwise set the end of the launch.
-    float rho = finite && a.probe_c > 0.0f ? probe_radius<WIN>(g, qx, qy, qz, a.k, a.probe_c) : rho0;
-    float rlo2 = 0.0f, rhi2 = -1.0f;  // the interval to subdivide (squared radii), rhi2 > 0
-    bool todo = finite;
-    for (int attempt = 0; attempt < 3 && __any_sync(FULL, todo); ++attempt) {
-        if (todo) {
-            todo = false;
-            const bool refine = rhi2 > 0.0f;
-            const float rmax = refine ? sqrtf(rhi2) : rho * rad_mul(NRAD - 1);
-            const int ulx = cell_of(__fsub_rn(qx, rmax), g.ox, g.inv_h);
-            const int uhx = cell_of(__fadd_rn(qx, rmax), g.ox, g.inv_h);
-            const int uly = cell_of(__fsub_rn(qy, rmax), g.oy, g.inv_h);
-            const int uhy = cell_of(__fadd_rn(qy, rmax), g.oy, g.inv_h);
-            const int ulz = cell_of(__fsub_rn(qz, rmax), g.oz, g.inv_h);
-            const int uhz = cell_of(__fadd_rn(qz, rmax), g.oz, g.inv_h);
-            float tau = certified_tau(g, qx, qy, qz, ulx, uhx, uly, uhy, ulz, uhz);
-            const float qm = fmaxf(fabsf(qx), fmaxf(fabsf(qy), fabsf(qz)));
-            {
-                const int cm = max(max(max(abs(ulx), abs(uhx + 1)), max(abs(uly), abs(uhy + 1))),
-                                   max(abs(ulz), abs(uhz + 1)));
-                eta = 0x1p-20f * (g.coord_scale + qm + (float)cm * g.h);
-            }
-            lx = max(ulx, WIN ? g.wlx : 0); hx = min(uhx, WIN ? g.whx : g.dimx - 1);
-            ly = max(uly, WIN ? g.wly : 0); hy = min(uhy, WIN ? g.why : g.dimy - 1);
-            lz = max(ulz, WIN ? g.wlz : 0); hz = min(uhz, WIN ? g.whz : g.dimz - 1);
-            const int64_t ncl = (int64_t)max(hx - lx + 1, 0) * max(hy - ly + 1, 0) * max(hz - lz + 1, 0);
-            const int64_t nrows = (int64_t)max(hy - ly + 1, 0) * max(hz - lz + 1, 0);
-            bool big = ncl > 4096 || nrows > 256 || (!g.dstart && ncl > 256);
-            if (DEL) {
-                const int vlx = cell_of(__fsub_rn(qx, rmax), dg.ox, dg.inv_h);
-                const int vhx = cell_of(__fadd_rn(qx, rmax), dg.ox, dg.inv_h);
-                const int vly = cell_of(__fsub_rn(qy, rmax), dg.oy, dg.inv_h);
-                const int vhy = cell_of(__fadd_rn(qy, rmax), dg.oy, dg.inv_h);
-                const int vlz = cell_of(__fsub_rn(qz, rmax), dg.oz, dg.inv_h);
-                const int vhz = cell_of(__fadd_rn(qz, rmax), dg.oz, dg.inv_h);
-                tau = fminf(tau, certified_tau(dg, qx, qy, qz, vlx, vhx, vly, vhy, vlz, vhz));
-                const int cm = max(max(max(abs(vlx), abs(vhx + 1)), max(abs(vly), abs(vhy + 1))),
-                                   max(abs(vlz), abs(vhz + 1)));
-                deta = 0x1p-20f * (dg.coord_scale + qm + (float)cm * dg.h);
-                dlx = max(vlx, WIN ? dg.wlx : 0); dhx = min(vhx, WIN ? dg.whx : dg.dimx - 1);
-                dly = max(vly, WIN ? dg.wly : 0); dhy = min(vhy, WIN ? dg.why : dg.dimy - 1);
-                dlz = max(vlz, WIN ? dg.wlz : 0); dhz = min(vhz, WIN ? dg.whz : dg.dimz - 1);
-                const int64_t dncl =
-                    (int64_t)max(dhx - dlx + 1, 0) * max(dhy - dly + 1, 0) * max(dhz - dlz + 1, 0);
-                const int64_t dnrows = (int64_t)max(dhy - dly + 1, 0) * max(dhz - dlz + 1, 0);
-                big = big || dncl > 4096 || dnrows > 256 || (!dg.dstart && dncl > 256);
-            }
-            fallback = false;
-            if (tau < 0.0f || big) {
-                fallback = true;
-            } else {
-                float t[NRAD];
-                int c[NRAD];
-#pragma unroll
-                for (int j = 0; j < NRAD; ++j) {
-                    const float r = rho * rad_mul(j);
-                    const float tr = refine ? rlo2 + (rhi2 - rlo2) * ((float)(j + 1) / (float)NRAD) : r * r;
-                    t[j] = fminf(tr, tau);
-                    c[j] = 0;
-                }
-                auto count = [&](uint32_t, const float4 p) {
-                    const float d = sqdist_pinned(qx, qy, qz, p.x, p.y, p.z);
-                    ++visits;
-#pragma unroll
-                    for (int j = 0; j < NRAD; ++j) c[j] += d <= t[j] ? 1 : 0;
-                };
-                if (g.dstart) for_rows<WIN>(g, qx, qy, qz, lx, hx, ly, hy, lz, hz, eta, t[NRAD - 1], count);
-                else for_box_points<WIN>(g, qx, qy, qz, lx, hx, ly, hy, lz, hz, eta, t[NRAD - 1], count);
-                if (DEL) {
-                    if (dg.dstart)
-                        for_rows<WIN>(dg, qx, qy, qz, dlx, dhx, dly, dhy, dlz, dhz, deta, t[NRAD - 1], count);
-                    else
-                        for_box_points<WIN>(dg, qx, qy, qz, dlx, dhx, dly, dhy, dlz, dhz, deta, t[NRAD - 1],
-                                            count);
-                }
-                int js = -1;
-#pragma unroll
-                for (int j = NRAD - 1; j >= 0; --j)
-                    if (c[j] >= k) js = j;
-                int cj = 0;
-                float tj = -1.0f, tl = -1.0f;
-#pragma unroll
-                for (int j = 0; j < NRAD; ++j) {
-                    if (j == js) { cj = c[j]; tj = t[j]; }
-                    if (j + 1 == js) tl = t[j];
-                }
-                if (js < 0 || cj > CAP) {
-                    fallback = true;
-                    // too few within the certified radii: widen (a wider box also
-                    // certifies further); too many: subdivide the jump or narrow
-                    const bool widen = js < 0;
-                    todo = true;
-                    if (!widen && js > 0 && !refine) {
-                        rlo2 = tl;
-                        rhi2 = tj;
-                    } else {
-                        rho = widen ? rho * 1.8f : rho * 0.7f;
-                        rhi2 = -1.0f;
-                    }
-                } else {
-                    m = cj;
-                    thr = tj;
-                }
-            }
+    const float mu = s / total, mv = __shfl_sync(FULL, mu, cv, G);
+    if constexpr (weighted) {
+        for (int j = 0; j < k; ++j) {
+            const float w = wt[j * CS];
+            const float du = (u[j * CS] - u0) - mu, dv = (v[j * CS] - v0) - mv;
+            // products weighted on the earlier coordinate, as in weighted_core
+            uu = __fmaf_rn(w * du, du, uu);
+            uv = cu == 2 ? __fmaf_rn(w * dv, du, uv) : __fmaf_rn(w * du, dv, uv);
+        }
+    } else {
+#pragma unroll 4
+        for (int j = 0; j < k; ++j) {
+            const float du = (u[j * CS] - u0) - mu, dv = (v[j * CS] - v0) - mv;
+            uu = __fmaf_rn(du, du, uu);
+            uv = __fmaf_rn(du, dv, uv);
         }
     }
-    if (m > 0) {
-        int w = 0;
-        auto collect = [&](uint32_t pos, const float4 p) {
+    uu = uu / total;
+    uv = uv / total;
+    return total;
+}
+
+// One unit of cnt <= 32 / G queries on one warp.  With DEL the search covers
+// the union of the main grid g and the grid dg of appended points (point j of
+// dg is g.m + j): both grids' boxes are walked, filtered by the smaller of
+// their certified taus, and list entries from dg carry DTAG.  Outputs may be
+// device memory or mapped host memory: rows and covariances are written as
+// contiguous blocks either way.
+template <int CAP, int G, int COV, bool WIN, bool DEL>
+__device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const float* __restrict__ q, int64_t n0,
+                                           int cnt, const TileArgs& a, float rho0, int32_t* __restrict__ idx,
+                                           float* __restrict__ d2, float* __restrict__ cov, unsigned char* smem) {
+    constexpr int SLOTS = lane_slots(CAP, G), WQ = 32 / G, NN = CAP / G;
+    constexpr int TB = SLOTS * G <= 64 ? 6 : 7;
+    constexpr uint32_t TAG = (1u << TB) - 1u;
+    constexpr int KMAX = CAP == 32 ? 24 : 32, ROUNDS = (WQ * KMAX + 31) / 32, CS = WQ + 1;
+    static_assert(4 * KMAX * CS <= SLOTS * 64 && 6 * WQ <= WQ * CAP, "coordinates and weights overlay the lists");
+    static_assert(SLOTS * G <= (1 << TB), "list slots must fit the key tag");
+    // k_knn_rest may be set up while the last blocks run (it waits for them)
+    cudaTriggerProgrammaticLaunchCompletion();
+    const int k = a.k;
+    const int lane = threadIdx.x, sub = lane & (G - 1);
+    float* const ld = reinterpret_cast<float*>(smem);
+    uint32_t* const lp = reinterpret_cast<uint32_t*>(smem + SLOTS * 32 * 4);
+    uint32_t* const kb = reinterpret_cast<uint32_t*>(smem + SLOTS * 32 * 8);
+    const int qi = lane / G;  // query of the unit
+    uint32_t* const kq = kb + qi * CAP;
+    const bool active = qi < cnt;
+    float qx = 0.0f, qy = 0.0f, qz = 0.0f;
+    if (active) {
+        const float* p = q + 3 * (n0 + qi);
+        qx = __ldg(p);
+        qy = __ldg(p + 1);
+        qz = __ldg(p + 2);
+    }
+    const bool finite = active && isfinite(qx) && isfinite(qy) && isfinite(qz);
+    uint32_t visits = 0;  // points of the rows this lane resolved
+
+    // ---- walk
+    float r2;
+    {
+        float r = rho0;
+        if (a.probe_c > 0.0f) r = probe_radius<G, WIN>(g, finite, qx, qy, qz, k, a.probe_c, sub);
+        r *= START;
+        r2 = fminf(r * r, 1e30f);
+    }
+    float lo2 = 0.0f, hi2 = -1.0f;  // squared radii known to hold too few / too many (hi2 > 0)
+    bool todo = finite, ok = false;
+    int w = 0, m = 0;
+    float t = -1.0f;
+    for (int attempt = 0; attempt < MAX_ATTEMPTS; ++attempt) {
+        if (!__any_sync(FULL, todo)) break;
+        GroupBox b, e;
+        float tt = -1.0f;
+        b.lx = b.ly = b.lz = e.lx = e.ly = e.lz = 0;
+        b.hx = b.hy = b.hz = e.hx = e.hy = e.hz = -1;
+        b.eta = e.eta = 0.0f;
+        if (todo) {
+            const float r = sqrtf(r2);
+            b = group_box<WIN>(g, qx, qy, qz, r);
+            float tau = b.tau;
+            bool big = b.big;
+            if (DEL) {
+                e = group_box<WIN>(dg, qx, qy, qz, r);
+                tau = fminf(tau, e.tau);
+                big = big || e.big;
+            }
+            tt = fminf(r2, tau);
+            if (big) todo = false;
+            else w = 0;
+        }
+        const bool act = todo && tt >= 0.0f;
+        auto keep = [&](uint32_t pos, const float4 p) {
             const float d = sqdist_pinned(qx, qy, qz, p.x, p.y, p.z);
-            ++visits;
-            if (d <= thr && w < CAP) {
-                posl[w * 32 + lane] = pos;
+            if (d <= tt) {
+                if (w < SLOTS) {
+                    ld[w * 32 + lane] = d;
+                    lp[w * 32 + lane] = pos;
+                }
                 ++w;
             }
         };
-        if (g.dstart) for_rows<WIN>(g, qx, qy, qz, lx, hx, ly, hy, lz, hz, eta, thr, collect);
-        else for_box_points<WIN>(g, qx, qy, qz, lx, hx, ly, hy, lz, hz, eta, thr, collect);
-        if (DEL) {
-            auto collect_d = [&](uint32_t pos, const float4 p) { collect(pos | DTAG, p); };
-            if (dg.dstart) for_rows<WIN>(dg, qx, qy, qz, dlx, dhx, dly, dhy, dlz, dhz, deta, thr, collect_d);
-            else for_box_points<WIN>(dg, qx, qy, qz, dlx, dhx, dly, dhy, dlz, dhz, deta, thr, collect_d);
-        }
-    }
-    __syncwarp();
-    uint32_t K[CAP];
-#pragma unroll
-    for (int s = 0; s < CAP; ++s) {
-        uint32_t key = 0xffffffffu;
-        if (s < m) {
-            const float4 p = pt_at<DEL>(g, dg, posl[s * 32 + lane]);
-            const float d = sqdist_pinned(qx, qy, qz, p.x, p.y, p.z);
-            key = ((__float_as_uint(d) << 1) & ~(uint32_t)(CAP - 1)) | (uint32_t)s;
-        }
-        K[s] = key;
-    }
-    const unsigned mmax = __reduce_max_sync(FULL, (unsigned)m);
-    if (mmax <= 16u) sort_regs<16>(K);
-    else if (CAP == 32 || mmax <= 32u) sort_regs<32>(K);
-    else sort_regs<CAP>(K);
-    bool amb = false;
-#pragma unroll
-    for (int r = 0; r + 1 < CAP; ++r) amb |= (r + 1 < m) && ((K[r] ^ K[r + 1]) < (uint32_t)CAP);
-    for (int pass = 0; amb && pass < CAP; ++pass) {
-        bool swapped = false;
-#pragma unroll
-        for (int r = 0; r + 1 < CAP; ++r) {
-            if (r + 1 < m && ((K[r] ^ K[r + 1]) < (uint32_t)CAP)) {
-                const u64 ka = slot_key<DEL>(g, dg, posl, (int)(K[r] & (CAP - 1)), lane, qx, qy, qz);
-                const u64 kb = slot_key<DEL>(g, dg, posl, (int)(K[r + 1] & (CAP - 1)), lane, qx, qy, qz);
-                if (kb < ka) {
-                    const uint32_t tmp = K[r];
-                    K[r] = K[r + 1];
-                    K[r + 1] = tmp;
-                    swapped = true;
-                }
+        group_walk<G, WIN>(g, act, qx, qy, qz, b.lx, b.hx, b.ly, b.hy, b.lz, b.hz, b.eta, tt, sub, visits, keep);
+        if (DEL)
+            group_walk<G, WIN>(dg, act, qx, qy, qz, e.lx, e.hx, e.ly, e.hy, e.lz, e.hz, e.eta, tt, sub, visits,
+                            [&](uint32_t pos, const float4 p) { keep(pos | DTAG, p); });
+        const uint32_t mm = group_sum<G>((uint32_t)w);
+        const bool over = (__ballot_sync(FULL, w > SLOTS) >> (lane & ~(G - 1)) & ((1u << G) - 1u)) != 0u;
+        if (todo) {
+            if (mm < (uint32_t)k) {  // widen; a wider box also certifies further
+                lo2 = r2;
+                const float f = fminf(fmaxf(1.7f * (float)k / (float)max(mm, 1u), 1.5f), 9.0f);
+                r2 = hi2 > 0.0f ? 0.5f * (lo2 + hi2) : fminf(fmaxf(r2, 1e-6f * g.h * g.h) * f, 1e30f);
+            } else if (over) {  // narrow
+                hi2 = tt;
+                r2 = lo2 > 0.0f ? 0.5f * (lo2 + hi2)
+                                : tt * fminf(fmaxf(1.6f * (float)k / (float)mm, 0.02f), 0.8f);
+            } else {
+                ok = true;
+                todo = false;
+                m = (int)mm;
+                t = tt;
             }
         }
-        amb = swapped;
     }
-    if (m > 0) {
-        int32_t* const irow = STG ? si + lane * k : idx + n * k;
-        float* const drow = STG ? sd + lane * k : d2 + n * k;
-        // rank-ordered positions, rewritten in place into the list's first k slots
-        uint32_t P[32];
+    if (!ok) w = 0;
+
+    // ---- selection
+    int u = w;  // entries of this lane that are kept
+    if (__any_sync(FULL, ok && m > CAP)) {
+        bool need = ok && m > CAP;
+        float lo = 0.0f, hi = t, sel = t;
+        int kept = m;
+        for (int round = 0; round < 10; ++round) {
+            if (!__any_sync(FULL, need)) break;
+            float th[4];
 #pragma unroll
-        for (int r = 0; r < 32; ++r)
-            if (r < k) P[r] = posl[(K[r] & (CAP - 1)) * 32 + lane];
-        // Each lane writes its own row, so every store instruction touches
-        // 32 rows; a row of 4j (2j) entries on a 16- (8-) byte aligned base is
-        // whole vectors, which takes a quarter (half) of the instructions.
-        const uintptr_t ab = STG ? reinterpret_cast<uintptr_t>(stg)
-                                 : reinterpret_cast<uintptr_t>(idx) | reinterpret_cast<uintptr_t>(d2);
-        const int vw = ((k & 3) == 0 && (ab & 15) == 0) ? 4 : (((k & 1) == 0 && (ab & 7) == 0) ? 2 : 1);
-        auto entry = [&](int r, int& iv, float& dv) {
-            posl[r * 32 + lane] = P[r];
-            const float4 p = pt_at<DEL>(g, dg, P[r]);
-            iv = (int)union_index<DEL>(g, P[r], p);
-            dv = sqdist_pinned(qx, qy, qz, p.x, p.y, p.z);
-        };
-        if (vw == 4) {
-#pragma unroll
-            for (int r = 0; r < 32; r += 4)
-                if (r < k) {
-                    int4 iv;
-                    float4 dv;
-                    entry(r, iv.x, dv.x);
-                    entry(r + 1, iv.y, dv.y);
-                    entry(r + 2, iv.z, dv.z);
-                    entry(r + 3, iv.w, dv.w);
-                    *reinterpret_cast<int4*>(irow + r) = iv;
-                    *reinterpret_cast<float4*>(drow + r) = dv;
+            for (int j = 0; j < 4; ++j)
+                th[j] = round == 0 ? t * (((float)k + (float)(CAP - k) * (0.25f * (float)j + 0.125f)) / (float)m)
+                                   : lo + (hi - lo) * (0.2f * (float)(j + 1));
+            uint32_t c = 0;
+            if (need)
+                for (int i = 0; i < w; ++i) {
+                    const float d = ld[i * 32 + lane];
+                    c += (d <= th[0] ? 1u : 0u) + (d <= th[1] ? 1u << 8 : 0u) + (d <= th[2] ? 1u << 16 : 0u) +
+                         (d <= th[3] ? 1u << 24 : 0u);
                 }
-        } else if (vw == 2) {
+            c = group_sum<G>(c);  // at most SLOTS * G < 256 each
+            if (need) {
+                bool found = false;
 #pragma unroll
-            for (int r = 0; r < 32; r += 2)
-                if (r < k) {
-                    int2 iv;
-                    float2 dv;
-                    entry(r, iv.x, dv.x);
-                    entry(r + 1, iv.y, dv.y);
-                    *reinterpret_cast<int2*>(irow + r) = iv;
-                    *reinterpret_cast<float2*>(drow + r) = dv;
+                for (int j = 0; j < 4; ++j) {
+                    const int cj = (int)(c >> (8 * j) & 255u);
+                    if (!found && cj >= k) {
+                        found = true;
+                        sel = th[j];
+                        kept = cj;
+                    }
+                    if (!found) lo = fmaxf(lo, th[j]);
                 }
-        } else {
+                if (found) hi = fminf(hi, sel);
+                need = !found || kept > CAP;
+            }
+        }
+        if (need) ok = false;  // more than CAP points at one distance
+        else if (ok) {
+            m = kept;
+            u = 0;
+            for (int i = 0; i < w; ++i) u += ld[i * 32 + lane] <= sel ? 1 : 0;
+            t = sel;
+        }
+        if (!ok) w = u = m = 0;
+    }
+
+    // ---- keys, in a compact row per query
+    {
+        int at = u;
 #pragma unroll
-            for (int r = 0; r < 32; ++r)
-                if (r < k) {
-                    int iv;
-                    float dv;
-                    entry(r, iv, dv);
-                    irow[r] = iv;
-                    drow[r] = dv;
-                }
+        for (int o = 1; o < G; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, at, o, G);
+            if (sub >= o) at += y;
         }
-    } else if (active && !finite) {
-        int32_t* const irow = STG ? si + lane * k : idx + n * k;
-        float* const drow = STG ? sd + lane * k : d2 + n * k;
-        for (int r = 0; r < k; ++r) {
-            irow[r] = -1;
-            drow[r] = INFINITY;
+        at -= u;
+        for (int i = 0; i < w; ++i) {
+            const float d = ld[i * 32 + lane];
+            if (d <= t) kq[at++] = ((__float_as_uint(d) << 1) & ~TAG) | (uint32_t)(i * G + sub);
         }
-        atomicOr(g.status, ST_NONFINITE);
-    }
-    unsigned fb = __ballot_sync(FULL, fallback);
-    const unsigned nvis = __reduce_add_sync(FULL, visits);
-    if (lane == 0) {
-        atomicAdd(&g.stats[0], (unsigned long long)cnt);
-        if (fb) atomicAdd(&g.stats[1], (unsigned long long)__popc(fb));
-        if (nvis) atomicAdd(&g.stats[3], (unsigned long long)nvis);
-    }
-    while (fb) {
-        const int f = __ffs(fb) - 1;
-        fb &= fb - 1u;
-        const float fx = __shfl_sync(FULL, qx, f), fy = __shfl_sync(FULL, qy, f),
-                    fz = __shfl_sync(FULL, qz, f);
-        float rho = rho0 * rad_mul(NRAD - 1);
-        SearchState<1> S;
-        state_reset(S);
-        const int sr = knn_search<1, DEL>(g, dg, fx, fy, fz, k, rho, S, pend, lane);
-        const bool ok = sr == SEARCH_OK;
-        if (!ok && lane == 0) atomicOr(g.status, sr == SEARCH_SHORT ? ST_SHORT : ST_SEARCH_LIMIT);
-        const int64_t nf = n0 + f;
-        if (lane < k) {
-            int32_t* const fi = STG ? si + f * k : idx + nf * k;
-            float* const fd = STG ? sd + f * k : d2 + nf * k;
-            fi[lane] = ok ? (int32_t)(uint32_t)S.L[0] : -1;
-            fd[lane] = ok ? __uint_as_float((uint32_t)(S.L[0] >> 32)) : INFINITY;
-        }
-    }
-    if (STG) {
-        __syncwarp();  // the staged rows of every lane, then one block per array
-        warp_copy_out(reinterpret_cast<uint32_t*>(idx + n0 * k), stg, cnt * k, lane);
-        warp_copy_out(reinterpret_cast<uint32_t*>(d2 + n0 * k), stg + 32 * k, cnt * k, lane);
-    }
-    if (COV && cov != nullptr) {
-        __syncwarp();  // orders the idx rows written by other lanes
-        float* const crow = STG ? sc + 6 * lane : cov + 6 * n;
-        if (m > 0) {  // neighbours straight from the cell-sorted copy, in rank order
-            auto get = [&](int j) { return pt_at<DEL>(g, dg, posl[j * 32 + lane]); };
-            if (a.ck.type != 0) weighted_core(get, a.ck, qx, qy, qz, k, a.eps, crow);
-            else cov_core(get, k, a.eps, crow);
-        } else if (active) {
-            cov_row_any<DEL>(g, dg, STG ? si + lane * k : idx + n * k, k, a, qx, qy, qz, crow);
-        }
-        if (STG) {
-            __syncwarp();
-            warp_copy_out(reinterpret_cast<uint32_t*>(cov + 6 * n0), stg + 64 * k, cnt * 6, lane);
-        }
+        for (int i = m + sub; i < CAP; i += G) kq[i] = 0xffffffffu;
     }
     __syncwarp();
+    uint32_t K[NN];
+    uint4* const kv = reinterpret_cast<uint4*>(kq + sub * NN);
+#pragma unroll
+    for (int i = 0; i < NN / 4; ++i) {
+        const uint4 v = kv[i];
+        K[4 * i] = v.x;
+        K[4 * i + 1] = v.y;
+        K[4 * i + 2] = v.z;
+        K[4 * i + 3] = v.w;
+    }
+    sort_group<NN, G>(K, sub);
+#pragma unroll
+    for (int i = 0; i < NN / 4; ++i) kv[i] = make_uint4(K[4 * i], K[4 * i + 1], K[4 * i + 2], K[4 * i + 3]);
+    bool amb = false;
+#pragma unroll
+    for (int i = 0; i + 1 < NN; ++i) amb |= (sub * NN + i + 1 < m) && ((K[i] ^ K[i + 1]) <= TAG);
+    {
+        const uint32_t nx = __shfl_down_sync(FULL, K[0], 1, G);
+        amb |= sub + 1 < G && (sub + 1) * NN < m && ((K[NN - 1] ^ nx) <= TAG);
+    }
+    __syncwarp();
+    const unsigned ambs = __ballot_sync(FULL, amb);
+    if (ambs) {
+        if (sub == 0 && (ambs >> lane & ((1u << G) - 1u)) != 0u) {
+            auto before = [&](uint32_t ka, uint32_t kc) {  // exact (d2, index) order of two entries
+                const int ia = (int)(ka & TAG), ic = (int)(kc & TAG);
+                const int sa = (ia / G) * 32 + lane + ia % G, sc = (ic / G) * 32 + lane + ic % G;
+                const float da = ld[sa], dc = ld[sc];
+                if (da != dc) return da < dc;
+                const uint32_t pa = lp[sa], pc = lp[sc];
+                return union_index<DEL>(g, pa, pt_at<DEL>(g, dg, pa)) < union_index<DEL>(g, pc, pt_at<DEL>(g, dg, pc));
+            };
+            for (int i = 1; i < m; ++i) {
+                const uint32_t x = kq[i];
+                int j = i;
+                while (j > 0 && ((kq[j - 1] ^ x) <= TAG) && before(x, kq[j - 1])) {
+                    kq[j] = kq[j - 1];
+                    --j;
+                }
+                kq[j] = x;
+            }
+        }
+        __syncwarp();
+    }
+
+    // ---- rows, one block per unit; the neighbours' coordinates go over the
+    // lists (at rank * (WQ + 1) + query: no bank conflicts, whether written
+    // rank by rank or read query by query)
+    const unsigned okm = __ballot_sync(FULL, ok), finm = __ballot_sync(FULL, finite);
+    const unsigned badm = finm & ~okm;
+    const bool with_cov = COV && cov != nullptr;
+    {
+        uint32_t* const d2b = reinterpret_cast<uint32_t*>(d2) + n0 * k;
+        int32_t* const ib = idx + n0 * k;
+        const uint32_t inv = (65536u + (uint32_t)k - 1u) / (uint32_t)k;  // e / k for e < 8 * 32
+        float nx[ROUNDS], ny[ROUNDS], nz[ROUNDS];
+        int to[ROUNDS];
+#pragma unroll
+        for (int it = 0; it < ROUNDS; ++it) {
+            const int e = lane + 32 * it;
+            to[it] = -1;
+            if (e < cnt * k) {
+                const int qe = (int)((uint32_t)e * inv >> 16), r = e - qe * k;
+                int iv = -1;
+                uint32_t dv = 0x7f800000u;  // +inf
+                if (okm >> (qe * G) & 1u) {
+                    const uint32_t tag = kb[qe * CAP + r] & TAG;
+                    const int at = (int)(tag / G) * 32 + qe * G + (int)(tag % G);
+                    dv = __float_as_uint(ld[at]);
+                    const uint32_t tp = lp[at];
+                    const float4 p = pt_at<DEL>(g, dg, tp);
+                    iv = (int)union_index<DEL>(g, tp, p);
+                    nx[it] = p.x;
+                    ny[it] = p.y;
+                    nz[it] = p.z;
+                    to[it] = r * CS + qe;
+                } else if (finm >> (qe * G) & 1u) {
+                    dv = UNANSWERED;
+                }
+                if (e == 0 && badm) dv |= UNIT_FLAG;
+                ib[e] = iv;
+                d2b[e] = dv;
+            }
+        }
+        if (with_cov) {
+            __syncwarp();  // the lists are done with
+#pragma unroll
+            for (int it = 0; it < ROUNDS; ++it)
+                if (to[it] >= 0) {
+                    ld[to[it]] = nx[it];
+                    ld[KMAX * CS + to[it]] = ny[it];
+                    ld[2 * KMAX * CS + to[it]] = nz[it];
+                }
+            __syncwarp();
+        }
+    }
+    visits = __reduce_add_sync(FULL, visits);
+    if (lane == 0) {
+        atomicAdd(&g.stats[3], (unsigned long long)visits);
+        if (badm) atomicAdd(&g.stats[1], (unsigned long long)(__popc(badm) / G));
+        if (__popc(finm) < cnt * G) atomicOr(g.status, ST_NONFINITE);
+    }
+    // ---- covariances
+    if (with_cov) {
+        float uu, uv;
+        const float total = group_moments<CS, KMAX, G, COV == 2>(ld + qi, a, qx, qy, qz, sub, uu, uv);
+        float* const sc = reinterpret_cast<float*>(kb);  // the keys are done with
+        const bool some = ok && total > 0.0f && isfinite(total);
+        const float nan = __uint_as_float(NAN_ROW);
+        if (sub < 3) {  // xx, xy; yy, yz; zz, xz
+            sc[6 * qi + (sub == 0 ? 0 : sub + 2 + (sub >> 1))] = some ? uu : nan;
+            sc[6 * qi + (sub == 0 ? 1 : sub == 1 ? 4 : 2)] = some ? uv : nan;
+        }
+        __syncwarp();
+        if (a.finish) {
+            if (sub == 0 && some) cov_regularise(sc + 6 * qi, a.eps);
+            __syncwarp();
+        }
+        for (int i = lane; i < 6 * cnt; i += 32) cov[6 * n0 + i] = sc[i];
+    }
 }
 
 // k > 32: the warp-cooperative search for each query of the tile in turn.
@@ -1212,97 +1383,79 @@ __device__ void warp_tile(const Grid& g, const Grid& dg, const float* __restrict
     }
 }
 
-template <int MODE, bool COV, bool WIN, bool DEL = false, bool STG = false>
-__device__ __forceinline__ void process_tile(const Grid& g, const Grid& dg, const float* __restrict__ q, int64_t n0,
-                                             int cnt, const TileArgs& a, float rho0,
-                                             int32_t* __restrict__ idx, float* __restrict__ d2,
-                                             float* __restrict__ cov, unsigned char* wsmem,
-                                             int lane) {
-    u64* pend = reinterpret_cast<u64*>(wsmem);
-    uint32_t* posl = reinterpret_cast<uint32_t*>(wsmem + 64 * sizeof(u64));
-    uint32_t* stg = STG ? reinterpret_cast<uint32_t*>(wsmem + warp_smem_bytes(MODE)) : nullptr;
-    if (MODE == 0)
-        lane_tile<32, COV, WIN, DEL, STG>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov, pend, posl, stg, lane);
-    else if (MODE == 1)
-        lane_tile<64, COV, WIN, DEL, STG>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov, pend, posl, stg, lane);
-    else
-        warp_tile<COV, DEL>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov, pend, lane);
+// Work items are issued last-first.  A spinning LiDAR scan stored ring by ring
+// with rising elevation ends with its farthest, sparsest points, whose units
+// cost the most; starting them first lets the cheap near-range units fill the
+// end of the launch.  (The order never changes a result.)  An item is one
+// block of the group search (CAP > 0) and one warp of the warp path (CAP = 0).
+template <int CAP>
+__device__ __forceinline__ int64_t work_item(int64_t items, int last_first) {
+    const int64_t w = CAP ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    return w >= items ? -1 : (last_first ? items - 1 - w : w);
 }
 
-template <int MODE, bool COV, bool WIN, bool STG = false>
-__global__ void __launch_bounds__(256, 2) k_knn(Grid g, const float* __restrict__ q, int64_t N,
-                                             int tile, TileArgs a, float rho0,
-                                             int32_t* __restrict__ idx, float* __restrict__ d2,
-                                             float* __restrict__ cov) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nwarps = blockDim.x >> 5;
-    // Tiles are issued last-first.  A spinning LiDAR scan stored ring by ring
-    // with rising elevation ends with its farthest, sparsest points, whose
-    // tiles cost the most; starting them first lets the cheap near-range
-    // tiles fill the end of the launch.  (The order never changes a result.)
-    const int64_t tiles = (N + tile - 1) / tile;
-    const int64_t w = (int64_t)blockIdx.x * nwarps + warp;
-    if (w >= tiles) return;
-    const int64_t t = a.last_first ? tiles - 1 - w : w;
-    const int64_t n0 = t * tile;
-    const int cnt = (int)min((int64_t)tile, N - n0);
-    process_tile<MODE, COV, WIN, false, STG>(g, g, q, n0, cnt, a, rho0, idx, d2, cov,
-                                             smem + (size_t)warp * warp_bytes(MODE, STG, a.k), lane);
-}
-
-// Batched form: one warp per (scan, tile) item of the scans' prefix-summed
-// tile table, found by a binary search over the table, items issued
-// last-first as in k_knn (the last scan's farthest tiles start first).  A
-// plain grid rather than a persistent loop over a device work counter: the
-// hardware block scheduler balances the load as well, and without the loop
-// state the kernel keeps k_knn's registers (a persistent version spilled at
-// the 128-register cap and ran 23 % slower than one launch over the same
-// queries concatenated).
-// At most 96 registers in the lane path with up to 32 survivors, which it
-// fits without spilling (left free, the compiler takes 111); the 64-survivor
-// and warp paths keep up to 128.
-template <int MODE, bool COV, bool WIN, bool STG = false>
-__global__ void __maxnreg__(MODE == 0 ? 96 : 128) k_knn_batch(Grid g, const ScanDesc* __restrict__ scans,
-                                                   int nscans, int64_t total_tiles, int tile,
-                                                   TileArgs a, float rho0) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nwarps = blockDim.x >> 5;
-    const int64_t w = (int64_t)blockIdx.x * nwarps + warp;
-    if (w >= total_tiles) return;
-    const int64_t item = a.last_first ? total_tiles - 1 - w : w;
+// The scan that owns work item `item` of a batch's tile table.
+__device__ __forceinline__ int scan_of_item(const ScanDesc* __restrict__ scans, int nscans, int64_t item) {
     int lo = 0, hi = nscans - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (scans[mid].tile0 <= item) lo = mid; else hi = mid - 1;
     }
-    const ScanDesc sd = scans[lo];
+    return lo;
+}
+
+template <int CAP, int G, int COV, bool WIN, bool DEL>
+__device__ __forceinline__ void process_tile(const Grid& g, const Grid& dg, const float* __restrict__ q, int64_t n0,
+                                             int cnt, const TileArgs& a, float rho0, int32_t* __restrict__ idx,
+                                             float* __restrict__ d2, float* __restrict__ cov) {
+    if constexpr (CAP > 0) {
+        __shared__ __align__(16) unsigned char smem[group_warp_smem(CAP, G)];
+        group_unit<CAP, G, COV, WIN, DEL>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov, smem);
+    } else {
+        __shared__ u64 pend[8][64];
+        warp_tile<COV != 0, DEL>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov, pend[threadIdx.x >> 5], threadIdx.x & 31);
+    }
+}
+
+// Threads of a block and, for the group search, blocks an SM should hold: 32
+// one-warp blocks (64 registers, 5 KB each), 24 with 64 sorted survivors.
+constexpr int block_threads(int cap) { return cap ? 32 : 256; }
+constexpr int block_target(int cap) { return cap == 32 ? 32 : cap == 64 ? 24 : 1; }
+
+template <int CAP, int G, int COV, bool WIN>
+__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
+    k_knn(Grid g, const float* __restrict__ q, int64_t N, int tile, TileArgs a, float rho0, int32_t* __restrict__ idx,
+          float* __restrict__ d2, float* __restrict__ cov) {
+    const int64_t t = work_item<CAP>((N + tile - 1) / tile, a.last_first);
+    if (t < 0) return;
+    const int64_t n0 = t * tile;
+    process_tile<CAP, G, COV, WIN, false>(g, g, q, n0, (int)min((int64_t)tile, N - n0), a, rho0, idx, d2, cov);
+}
+
+// Batched form: work items are the (scan, tile) pairs of the scans'
+// prefix-summed tile table, found by a binary search over the table.
+template <int CAP, int G, int COV, bool WIN>
+__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
+    k_knn_batch(Grid g, const ScanDesc* __restrict__ scans, int nscans, int64_t total_tiles, int tile, TileArgs a,
+                float rho0) {
+    const int64_t item = work_item<CAP>(total_tiles, a.last_first);
+    if (item < 0) return;
+    const ScanDesc sd = scans[scan_of_item(scans, nscans, item)];
     const int64_t n0 = (item - sd.tile0) * tile;
-    const int cnt = (int)min((int64_t)tile, sd.n - n0);
-    process_tile<MODE, COV, WIN, false, STG>(g, g, sd.q, n0, cnt, a, rho0, sd.idx, sd.d2, sd.cov,
-                                             smem + (size_t)warp * warp_bytes(MODE, STG, a.k), lane);
+    process_tile<CAP, G, COV, WIN, false>(g, g, sd.q, n0, (int)min((int64_t)tile, sd.n - n0), a, rho0, sd.idx, sd.d2,
+                                          sd.cov);
 }
 
 // Search over a map grown by appended points: the main grid g and the
 // appended-points grid dg as one map (indices of dg's points follow g's).
-// Same tiling and tile order as k_knn.
-template <int MODE, bool COV, bool WIN>
-__global__ void __launch_bounds__(256, 2) k_knn_union(Grid g, Grid dg, const float* __restrict__ q, int64_t N,
-                                                   int tile, TileArgs a, float rho0,
-                                                   int32_t* __restrict__ idx, float* __restrict__ d2,
-                                                   float* __restrict__ cov) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nwarps = blockDim.x >> 5;
-    const int64_t tiles = (N + tile - 1) / tile;
-    const int64_t w = (int64_t)blockIdx.x * nwarps + warp;
-    if (w >= tiles) return;
-    const int64_t t = a.last_first ? tiles - 1 - w : w;
+template <int CAP, int G, int COV, bool WIN>
+__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
+    k_knn_union(Grid g, Grid dg, const float* __restrict__ q, int64_t N, int tile, TileArgs a, float rho0,
+                int32_t* __restrict__ idx, float* __restrict__ d2, float* __restrict__ cov) {
+    const int64_t t = work_item<CAP>((N + tile - 1) / tile, a.last_first);
+    if (t < 0) return;
     const int64_t n0 = t * tile;
-    const int cnt = (int)min((int64_t)tile, N - n0);
-    process_tile<MODE, COV, WIN, true>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov,
-                                       smem + (size_t)warp * warp_smem_bytes(MODE), lane);
+    process_tile<CAP, G, COV, WIN, true>(g, dg, q, n0, (int)min((int64_t)tile, N - n0), a, rho0, idx, d2, cov);
 }
 
 __global__ void k_cov(Grid g, const int32_t* __restrict__ idx, int64_t N, int k, float eps,
@@ -1312,71 +1465,31 @@ __global__ void k_cov(Grid g, const int32_t* __restrict__ idx, int64_t N, int k,
     cov_row(g, idx + n * k, 1, k, eps, cov + 6 * n, true);
 }
 
-template <typename K>
-cudaError_t allow_smem(K kern) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+// The search kernel of FORM (0 one scan, 1 batched, 2 union) and WIN for mode
+// = search_mode(k) and `group` lanes per query of the group search; cov 0 none,
+// 1 plain, 2 weighted by a kernel descriptor.  (Weighted covariances have
+// kernels of their own: the descriptors' code beside the plain sums cost the
+// plain search 10 % in instruction fetches.)
+template <int FORM, bool WIN, int CAP, int G, int COV>
+void* form_kernel() {
+    if constexpr (FORM == 0) return (void*)k_knn<CAP, G, COV, WIN>;
+    else if constexpr (FORM == 1) return (void*)k_knn_batch<CAP, G, COV, WIN>;
+    else return (void*)k_knn_union<CAP, G, COV, WIN>;
 }
-
-// The search kernel for (mode, covariance, batched) of this window variant.
-template <bool WIN>
-void* knn_kernel(int mode, bool with_cov, bool batch, bool stage = false) {
-    // outputs in host memory: the staged lane-path kernels
-    if (stage && mode < 2) {
-        if (batch && with_cov)
-            return mode == 0 ? (void*)k_knn_batch<0, true, WIN, true> : (void*)k_knn_batch<1, true, WIN, true>;
-        if (batch)
-            return mode == 0 ? (void*)k_knn_batch<0, false, WIN, true> : (void*)k_knn_batch<1, false, WIN, true>;
-        if (with_cov) return mode == 0 ? (void*)k_knn<0, true, WIN, true> : (void*)k_knn<1, true, WIN, true>;
-    }
-#define PC_PICK(M, C) (batch ? (void*)k_knn_batch<M, C, WIN> : (void*)k_knn<M, C, WIN>)
-    switch (mode * 2 + (with_cov ? 1 : 0)) {
-        case 0: return PC_PICK(0, false);
-        case 1: return PC_PICK(0, true);
-        case 2: return PC_PICK(1, false);
-        case 3: return PC_PICK(1, true);
-        case 4: return PC_PICK(2, false);
-        default: return PC_PICK(2, true);
-    }
-#undef PC_PICK
+template <int FORM, bool WIN, int CAP, int G>
+void* form_kernel(int cov) {
+    if (cov == 0) return form_kernel<FORM, WIN, CAP, G, 0>();
+    if (CAP == 0 || cov == 1) return form_kernel<FORM, WIN, CAP, G, 1>();
+    return form_kernel<FORM, WIN, CAP, G, CAP == 0 ? 1 : 2>();
 }
-
-// The union search kernel for (mode, covariance) of this window variant.
-template <bool WIN>
-void* knn_union_kernel(int mode, bool with_cov) {
-    switch (mode * 2 + (with_cov ? 1 : 0)) {
-        case 0: return (void*)k_knn_union<0, false, WIN>;
-        case 1: return (void*)k_knn_union<0, true, WIN>;
-        case 2: return (void*)k_knn_union<1, false, WIN>;
-        case 3: return (void*)k_knn_union<1, true, WIN>;
-        case 4: return (void*)k_knn_union<2, false, WIN>;
-        default: return (void*)k_knn_union<2, true, WIN>;
-    }
+template <int FORM, bool WIN, int CAP>
+void* form_kernel(int cov, int group) {
+    return group == 4 ? form_kernel<FORM, WIN, CAP, 4>(cov) : form_kernel<FORM, WIN, CAP, 8>(cov);
 }
-
-template <bool WIN>
-cudaError_t allow_union_smem() {
-    cudaError_t e = cudaSuccess;
-    for (int mode = 0; mode < 3; ++mode)
-        for (int c = 0; c < 2; ++c)
-            if ((e = allow_smem(knn_union_kernel<WIN>(mode, c != 0))) != cudaSuccess) return e;
-    return cudaSuccess;
-}
-
-// Opts every search kernel of this window variant into large dynamic
-// shared memory.
-template <bool WIN>
-cudaError_t allow_all_smem() {
-    cudaError_t e = cudaSuccess;
-    for (int mode = 0; mode < 3; ++mode)
-        for (int c = 0; c < 2; ++c)
-            for (int b = 0; b < 2; ++b)
-                if ((e = allow_smem(knn_kernel<WIN>(mode, c != 0, b != 0))) != cudaSuccess) return e;
-    for (int mode = 0; mode < 2; ++mode)
-        for (int c = 0; c < 2; ++c)
-            for (int b = 0; b < 2; ++b)
-                if ((e = allow_smem(knn_kernel<WIN>(mode, c != 0, b != 0, true))) != cudaSuccess) return e;
-    return cudaSuccess;
+template <int FORM, bool WIN>
+void* knn_kernel(int mode, int cov, int group) {
+    if (mode == 2) return form_kernel<FORM, WIN, 0, 1>(cov);
+    return mode == 0 ? form_kernel<FORM, WIN, 32>(cov, group) : form_kernel<FORM, WIN, 64>(cov, group);
 }
 
 }  // namespace
-

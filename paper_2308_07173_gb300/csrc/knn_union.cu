@@ -5,6 +5,4 @@
 // window variant.  Both compile in parallel with the other search units.
 #include "knn_kernels.cuh"
 
-void* pc_knn_union_kernel(int mode, bool with_cov) { return knn_union_kernel<false>(mode, with_cov); }
-
-cudaError_t pc_knn_union_attrs() { return allow_union_smem<false>(); }
+void* pc_knn_kernel_union(int mode, int cov, int group) { return knn_kernel<2, false>(mode, cov, group); }

@@ -2,6 +2,6 @@
 // window's boundary cells of either grid test each point against the window.
 #include "knn_kernels.cuh"
 
-void* pc_knn_union_kernel_win(int mode, bool with_cov) { return knn_union_kernel<true>(mode, with_cov); }
-
-cudaError_t pc_knn_union_win_attrs() { return allow_union_smem<true>(); }
+void* pc_knn_kernel_union_win(int mode, int cov, int group) {
+    return knn_kernel<2, true>(mode, cov, group);
+}

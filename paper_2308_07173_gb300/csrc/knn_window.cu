@@ -3,8 +3,8 @@
 // cells test each point against the window box.
 #include "knn_kernels.cuh"
 
-void* pc_knn_kernel_win(int mode, bool with_cov, bool batch, bool stage) {
-    return knn_kernel<true>(mode, with_cov, batch, stage);
+void* pc_knn_kernel_win(int form, int mode, int cov, int group) {
+    return form == 2   ? pc_knn_kernel_union_win(mode, cov, group)
+           : form == 1 ? pc_knn_kernel_batch_win(mode, cov, group)
+                       : knn_kernel<0, true>(mode, cov, group);
 }
-
-cudaError_t pc_knn_win_attrs() { return allow_all_smem<true>(); }

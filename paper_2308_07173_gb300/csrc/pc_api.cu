@@ -196,9 +196,8 @@ static pc_status build_target_internal(const float* xyz, int64_t M, const pc_bui
 // The search over the target as it stands: its grid, or its grid and the
 // delta grid of appended points searched as one map.
 static pc_status launch_search(pc_target_s* t, const float* q, int64_t N, int k, float eps, int32_t* idx,
-                               float* d2, float* cov, cudaStream_t st, bool stage = false) {
-    if (!t->delta) return pc_from_cuda(pc_launch_knn(t, q, N, k, eps, idx, d2, cov, pc_rho0(t, k), st, stage));
-    return pc_from_cuda(pc_launch_knn_union(t, q, N, k, eps, idx, d2, cov, pc_rho0(t, k), st));
+                               float* d2, float* cov, cudaStream_t st, bool host_cov = false) {
+    return pc_from_cuda(pc_launch_knn(t, q, N, k, eps, idx, d2, cov, pc_rho0(t, k), st, host_cov));
 }
 
 // The device address of page-locked host memory mapped into the device's
@@ -216,7 +215,7 @@ static void* mapped_host(const void* p) {
 // The address kernels use for p: p itself for device (or managed) memory,
 // the device address of mapped page-locked host memory (and *host = true),
 // null for anything else.
-static void* device_view(const void* p, bool* host) {
+static void* device_view(const void* p, bool* host = nullptr) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
@@ -224,7 +223,7 @@ static void* device_view(const void* p, bool* host) {
     }
     if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) return const_cast<void*>(p);
     if (a.type == cudaMemoryTypeHost && a.devicePointer) {
-        *host = true;
+        if (host) *host = true;
         return a.devicePointer;
     }
     return nullptr;
@@ -397,7 +396,8 @@ pc_status pc_knn_cov_host(pc_target t, const float* q_host, int64_t N, int k, fl
     cudaStream_t st = (cudaStream_t)s;
     // Page-locked outputs (k <= 32, no appended points): the search writes
     // them in place, each warp's rows as one block, so the transfer runs
-    // during the search; a page-locked q is read in place too.
+    // during the search; a page-locked q is read in place too.  (The warp
+    // path writes row by row, so wider k keeps the staged copies.)
     void* const mi = (k <= 32 && !t->delta) ? mapped_host(idx_host) : nullptr;
     void* const md = mi ? mapped_host(d2_host) : nullptr;
     void* const mc = md ? mapped_host(cov_host) : nullptr;
@@ -486,16 +486,12 @@ pc_status pc_batch_plan(pc_target t, const pc_scan* scans, int n_scans, int k, f
     b->k = k;
     b->eps = eps;
     b->with_cov = sh.any_cov;
-    b->host_out = sh.host_out;
+    b->host_cov = sh.host_cov;
     b->tile = sh.tile;
     b->warps = sh.warps;
-    b->max_n = sh.max_n;
     b->total_tiles = sh.tiles;
-    int64_t queries = 0;
-    for (int i = 0; i < n_scans; ++i) queries += scans[i].n;
-    b->total_queries = queries;
-    cudaError_t e = pc_knn_prepare();
-    if (e == cudaSuccess) e = cudaMalloc(&b->scans_dev, sizeof(ScanDesc) * n_scans);
+    b->total_queries = sh.queries;
+    cudaError_t e = cudaMalloc(&b->scans_dev, sizeof(ScanDesc) * n_scans);
     if (e == cudaSuccess)
         e = cudaMemcpy(b->scans_dev, hs.data(), sizeof(ScanDesc) * n_scans, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -518,9 +514,9 @@ pc_status pc_batch_run(pc_batch b, pc_stream s) {
     cudaStream_t st = (cudaStream_t)s;
     const float rho0 = pc_rho0(b->t, b->k);
     if (st == nullptr)  // the legacy stream cannot be captured: launch directly
-        return pc_from_cuda(pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans, b->max_n,
-                                                b->total_tiles, b->tile, b->warps, b->k, b->eps, b->with_cov,
-                                                rho0, st, b->host_out));
+        return pc_from_cuda(pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans,
+                                                b->total_tiles, b->total_queries, b->tile, b->warps, b->k, b->eps,
+                                                b->with_cov, b->host_cov, rho0, st));
     if (!b->exec || b->captured_on != st) {
         if (b->exec) cudaGraphExecDestroy(b->exec);
         if (b->graph) cudaGraphDestroy(b->graph);
@@ -528,8 +524,9 @@ pc_status pc_batch_run(pc_batch b, pc_stream s) {
         b->graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return pc_from_cuda(e);
-        cudaError_t e2 = pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans, b->max_n, b->total_tiles,
-                                             b->tile, b->warps, b->k, b->eps, b->with_cov, rho0, st, b->host_out);
+        cudaError_t e2 = pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans, b->total_tiles,
+                                             b->total_queries, b->tile, b->warps, b->k, b->eps, b->with_cov,
+                                             b->host_cov, rho0, st);
         e = cudaStreamEndCapture(st, &b->graph);
         if (e2 != cudaSuccess) e = e2;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
@@ -558,12 +555,12 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
     if (t->delta) return PC_ERR_INVALID_ARG;  // appended points: pc_target_compact first
     if ((int64_t)k > t->g.m) return PC_ERR_K_GT_M;
     BatchShape sh;
-    sh.tile = std::min(std::max(t->tune.tile, 1), 32);
+    sh.queries = 0;
+    for (int i = 0; i < n_scans; ++i) sh.queries += std::max<int64_t>(scans[i].n, 0);
+    sh.tile = pc_search_tile(t, k, sh.queries);
     sh.warps = std::min(std::max(t->tune.warps, 1), 8);
     sh.tiles = 0;
-    sh.max_n = 0;
-    sh.any_cov = false;
-    sh.host_out = false;
+    sh.any_cov = sh.host_cov = false;
     for (int i = 0; i < n_scans; ++i) {
         const pc_scan& sc = scans[i];
         if (sc.n < 0) return PC_ERR_INVALID_ARG;
@@ -571,13 +568,12 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
         void *idx = sc.idx_dev, *d2 = sc.d2_dev, *cov = sc.cov_dev;
         if (sc.n > 0) {
             if (!sc.q_dev || !sc.idx_dev || !sc.d2_dev) return PC_ERR_INVALID_ARG;
-            bool host_q = false;
-            q = device_view(sc.q_dev, &host_q);
-            idx = device_view(sc.idx_dev, &sh.host_out);
-            d2 = device_view(sc.d2_dev, &sh.host_out);
+            q = device_view(sc.q_dev);
+            idx = device_view(sc.idx_dev);
+            d2 = device_view(sc.d2_dev);
             if (!q || !idx || !d2) return PC_ERR_BAD_POINTER;
             if (sc.cov_dev) {
-                if (!(cov = device_view(sc.cov_dev, &sh.host_out))) return PC_ERR_BAD_POINTER;
+                if (!(cov = device_view(sc.cov_dev, &sh.host_cov))) return PC_ERR_BAD_POINTER;
                 sh.any_cov = true;
             }
         }
@@ -588,7 +584,6 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
         table[i].cov = static_cast<float*>(cov);
         table[i].tile0 = sh.tiles;
         sh.tiles += (sc.n + sh.tile - 1) / sh.tile;
-        sh.max_n = std::max<int64_t>(sh.max_n, sc.n);
     }
     *shape = sh;
     return PC_OK;
@@ -620,8 +615,8 @@ pc_status pc_batch_run_scratch(pc_target t, const pc_scan* scans, int n_scans, i
     cudaError_t e = cudaMemcpyAsync(table, hs.data(), sizeof(ScanDesc) * n_scans,
                                     cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
-        e = pc_launch_knn_batch(t, t->g, t->ck, table, n_scans, sh.max_n, sh.tiles, sh.tile, sh.warps, k, eps,
-                                sh.any_cov, pc_rho0(t, k), st, sh.host_out);
+        e = pc_launch_knn_batch(t, t->g, t->ck, table, n_scans, sh.tiles, sh.queries, sh.tile, sh.warps, k, eps,
+                                sh.any_cov, sh.host_cov, pc_rho0(t, k), st);
     return pc_from_cuda(e);
 }
 

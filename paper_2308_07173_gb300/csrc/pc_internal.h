@@ -21,6 +21,16 @@ struct CovKernel {
     float ox, oy, oz;
 };
 
+// What a search launch passes to its kernels besides the grid and buffers.
+struct TileArgs {
+    int k;
+    float eps;
+    int last_first;  // issue tiles from the end of the query array
+    CovKernel ck;    // kernel-descriptor weights; type 0: the plain covariance
+    int finish;      // group search: regularise in place (outputs in host memory) instead of in k_knn_rest
+    float probe_c;   // > 0: every query estimates its own starting radius (probe_radius)
+};
+
 // One scan of a batched launch, as the batched kernel reads it from the scan table.
 struct ScanDesc {
     const float* q;
@@ -71,12 +81,11 @@ struct pc_batch_s {
     pc_target_s* t;
     pcdev::Grid g;  // the target's view when planned (window included)
     CovKernel ck;   // and its covariance weights
-    int64_t max_n;  // largest scan
     int n_scans;
     int k;
     float eps;
     bool with_cov;
-    bool host_out;  // outputs in mapped host memory: the staged kernel
+    bool host_cov;  // some covariance output is mapped host memory
     int tile;
     int warps;
     int64_t total_tiles;
@@ -112,26 +121,34 @@ size_t pc_scan_temp_words(int64_t n);
 cudaError_t pc_scan_exclusive(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total_dev,
                               uint32_t* temp, cudaStream_t s);
 
-// knn_window.cu: the window variant of the search kernels
-void* pc_knn_kernel_win(int mode, bool with_cov, bool batch, bool stage = false);
-cudaError_t pc_knn_win_attrs();
+// The search kernels' translation units (whole-map / window variants, with or
+// without appended points): form 0 one scan, 1 batched, 2 union; group: lanes
+// per query of the group search (k <= 32).
+void* pc_knn_kernel_win(int form, int mode, int cov, int group);
+void* pc_knn_kernel_batch(int mode, int cov, int group);
+void* pc_knn_kernel_batch_win(int mode, int cov, int group);
+void* pc_knn_kernel_union(int mode, int cov, int group);
+void* pc_knn_kernel_union_win(int mode, int cov, int group);
 
-// knn_cov.cu.  stage: the outputs are host-mapped memory; each warp stages
-// its tile's rows in shared memory and writes them as whole blocks (lane
-// path with covariance; the warp path, k > 32, writes its rows directly).
+// knn_cov.cu.  Outputs may be device or mapped page-locked host memory.
 cudaError_t pc_launch_knn(const pc_target_s* t, const float* q, int64_t N, int k, float eps,
-                          int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s, bool stage = false);
-cudaError_t pc_launch_knn_union(const pc_target_s* t, const float* q, int64_t N, int k, float eps,
-                                int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s);
-// Opts the search kernels into large shared memory on the current device
-// (once; call outside any stream capture).
-cudaError_t pc_knn_prepare();
+                          int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s, bool host_cov = false);
+// Queries of one work item of a search over n queries (k <= 32: a unit of the
+// group search; else the tune's tile).
+int pc_search_tile(const pc_target_s* t, int k, int64_t n);
 cudaError_t pc_launch_cov(const pc_target_s* t, const int32_t* idx, int64_t N, int k, float eps,
                           float* cov, cudaStream_t s);
 cudaError_t pc_launch_knn_batch(const pc_target_s* t, const pcdev::Grid& g, const CovKernel& ck,
-                                const ScanDesc* scans_dev, int nscans, int64_t max_n,
-                                int64_t total_tiles, int tile, int warps, int k, float eps,
-                                bool with_cov, float rho0, cudaStream_t s, bool stage = false);
+                                const ScanDesc* scans_dev, int nscans, int64_t total_tiles, int64_t queries,
+                                int tile, int warps, int k, float eps, bool with_cov, bool host_cov, float rho0,
+                                cudaStream_t s);
+
+// knn_rest.cu: the queries that a group search (k <= 32) over the same
+// arguments left unanswered; dg: the appended points' grid, or null.
+cudaError_t pc_launch_rest(const pcdev::Grid& g, const pcdev::Grid* dg, const float* q, int64_t N, int tile,
+                           const TileArgs& a, float rho0, int32_t* idx, float* d2, float* cov, cudaStream_t s);
+cudaError_t pc_launch_rest_batch(const pcdev::Grid& g, const ScanDesc* scans_dev, int nscans, int64_t total_tiles,
+                                 int64_t queries, int tile, const TileArgs& a, float rho0, cudaStream_t s);
 
 // gicp.cu
 size_t pc_gicp_work_size();
@@ -141,13 +158,6 @@ cudaError_t pc_launch_gicp_linearize(const pc_target_s* t, const float* map_cov,
                                      float r0, float r0d, cudaStream_t s);
 cudaError_t pc_launch_gicp_update(const double* lin, float lambda, float* pose, double* xi,
                                   cudaStream_t s);
-
-// knn_union.cu / knn_union_win.cu: the search kernels over the main grid
-// plus the delta grid (whole-map and window variants)
-void* pc_knn_union_kernel(int mode, bool with_cov);
-cudaError_t pc_knn_union_attrs();
-void* pc_knn_union_kernel_win(int mode, bool with_cov);
-cudaError_t pc_knn_union_win_attrs();
 
 // delta.cu: covariances and packing over the main grid plus the delta grid
 cudaError_t pc_launch_cov_union(const pc_target_s* t, const int32_t* idx, int64_t N, int k, float eps,
@@ -161,10 +171,10 @@ float pc_probe_c(const pc_target_s* t);
 // Launch shape of a batched call over caller-provided scans.
 struct BatchShape {
     int64_t tiles;  // work items (tiles of `tile` queries) over all scans; 0: nothing to do
-    int64_t max_n;  // largest scan
     int tile, warps;
+    int64_t queries;
     bool any_cov;   // some scan asks for covariances
-    bool host_out;  // some output is mapped page-locked host memory (staged block writes)
+    bool host_cov;  // into mapped host memory
 };
 // Argument checks and scan table shared by pc_batch_plan,
 // pc_batch_run_scratch and pc_batch_run_noalloc; fills table[0, n_scans)

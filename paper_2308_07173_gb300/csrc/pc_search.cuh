@@ -50,6 +50,18 @@ __device__ __forceinline__ float certified_tau(const Grid& g, float qx, float qy
     return (Rs * Rs) * (1.0f - 0x1p-20f);
 }
 
+// Lower bound on the squared distance from q to cell (cx, cy, cz): the gaps
+// on each axis less the rounding margin eta.
+__device__ __forceinline__ float box_gap2(const Grid& g, float qx, float qy, float qz, int cx, int cy, int cz,
+                                          float eta) {
+    auto gap = [&](float q, float o, int c) {
+        const float lo = o + (float)c * g.h, hi = o + (float)(c + 1) * g.h;
+        return fmaxf(fmaxf(fmaxf(lo - q, q - hi), 0.0f) - eta, 0.0f);
+    };
+    const float gx = gap(qx, g.ox, cx), gy = gap(qy, g.oy, cy), gz = gap(qz, g.oz, cz);
+    return gz * gz + gy * gy + gx * gx;
+}
+
 // Visit every point of the cell box [l, h] (clamped to the grid) whose
 // cell can hold a point within sqrt(tmax) of q, as f(position, point).
 // Rows along x are pruned by a conservative lower bound (the eta margin of
