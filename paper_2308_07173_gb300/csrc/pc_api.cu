@@ -89,54 +89,35 @@ pc_status read_and_clear_status(pc_target_s* t, cudaStream_t s) {
 
 // First search radius per k: the 75th percentile of the k-th neighbour
 // distance over up to 1024 target points used as queries.  It only sets
-// where the widening search starts; results never depend on it.
+// where the widening search starts; results never depend on it.  The sample
+// and the percentiles are taken on the device (grid_build.cu): one copy of 66
+// floats comes back.
 pc_status calibrate_rho(pc_target_s* t, cudaStream_t s) {
     const int64_t M = t->g.m;
     const int kc = (int)std::min<int64_t>(64, M);
     const int64_t S = std::min<int64_t>(M, 1024);
-    const int64_t step = M / S;
-    float* q = nullptr;
-    int32_t* idx = nullptr;
-    float* d2 = nullptr;
-    cudaError_t e = cudaMalloc(&q, sizeof(float) * 3 * S);
-    if (e == cudaSuccess) e = cudaMalloc(&idx, sizeof(int32_t) * S * kc);
-    if (e == cudaSuccess) e = cudaMalloc(&d2, sizeof(float) * S * kc);
-    std::vector<float> hd((size_t)S * kc);
-    if (e == cudaSuccess)
-        e = cudaMemcpy2DAsync(q, 3 * sizeof(float), t->xyz, sizeof(float4) * step, 3 * sizeof(float),
-                              S, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = pc_launch_knn(t, q, S, kc, -1.0f, idx, d2, nullptr, t->g.h, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(hd.data(), d2, sizeof(float) * S * kc, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (q) cudaFree(q);
-    if (idx) cudaFree(idx);
-    if (d2) cudaFree(d2);
+    float* buf = nullptr;  // sample points, distances, hints, indices
+    const size_t words = (size_t)S * 3 + (size_t)S * kc * 2 + 66;
+    cudaError_t e = cudaMalloc(&buf, words * sizeof(float));
     if (e != cudaSuccess) return pc_from_cuda(e);
-    read_and_clear_status(t, s);  // a capped search here only skips that sample
-    cudaMemsetAsync(reinterpret_cast<char*>(t->status) + 32, 0, 32, s);
-    cudaStreamSynchronize(s);
-    std::vector<float> col;
-    for (int kk = 0; kk < 64; ++kk) {
-        t->rho_hint[kk] = 0.0f;
-        if (kk >= kc) continue;
-        col.clear();
-        for (int64_t n = 0; n < S; ++n) {
-            const float v = hd[(size_t)n * kc + kk];
-            if (std::isfinite(v)) col.push_back(std::sqrt(v));
-        }
-        if (col.empty()) continue;
-        const size_t pos = (col.size() * 3) / 4;
-        std::nth_element(col.begin(), col.begin() + pos, col.end());
-        t->rho_hint[kk] = col[pos];
-        // spread of the distances at k = min(kc, 16): a map whose density
-        // varies widely (a p90 / p25 above 1.55) gets per-query starting radii
-        if (kk == std::min(kc, 16) - 1) {
-            std::sort(col.begin(), col.end());
-            const float p25 = col[col.size() / 4], p90 = col[(col.size() * 9) / 10];
-            t->uneven = p25 > 0.0f && p90 > 1.55f * p25 ? 1 : 0;
-        }
-    }
+    float* const q = buf;
+    float* const d2 = q + 3 * S;
+    float* const hints = d2 + S * kc;
+    int32_t* const idx = reinterpret_cast<int32_t*>(hints + 66);
+    float h[66];
+    e = pc_launch_sample(t, S, q, s);
+    if (e == cudaSuccess) e = pc_launch_knn(t, q, S, kc, -1.0f, idx, d2, nullptr, t->g.h, s);
+    if (e == cudaSuccess) e = pc_launch_rho_hints(d2, (int)S, kc, hints, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, hints, sizeof(h), cudaMemcpyDeviceToHost, s);
+    // the status word and statistics start clean (a capped search here only skips that sample)
+    if (e == cudaSuccess) e = cudaMemsetAsync(t->status, 0, 64, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);
+    cudaFree(buf);
+    if (e != cudaSuccess || e2 != cudaSuccess) return pc_from_cuda(e != cudaSuccess ? e : e2);
+    std::memcpy(t->rho_hint, h, 64 * sizeof(float));
+    // spread of the distances at k = min(kc, 16): a map whose density varies
+    // widely (a p90 / p25 above 1.55) gets per-query starting radii
+    t->uneven = h[64] > 0.0f && h[65] > 1.55f * h[64] ? 1 : 0;
     return PC_OK;
 }
 

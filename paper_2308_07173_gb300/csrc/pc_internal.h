@@ -114,6 +114,12 @@ inline void pc_clear_window(pcdev::Grid& g) {
 pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& o, cudaStream_t s,
                         pc_target_s* t);
 void pc_free_grid(pc_target_s* t);
+// Every (M / n)-th point of the target in caller order, to q [n, 3].
+cudaError_t pc_launch_sample(const pc_target_s* t, int64_t n, float* q, cudaStream_t s);
+// Over n <= 1024 rows of kc <= 64 squared distances: out[k] = the 75th
+// percentile of column k's finite distances (0: none), out[64], out[65] = the
+// 25th and 90th of column min(kc, 16) - 1.
+cudaError_t pc_launch_rho_hints(const float* d2, int n, int kc, float* out, cudaStream_t s);
 size_t pc_sort_temp_words(int64_t n);
 cudaError_t pc_radix_sort_pairs(unsigned long long** keys, uint32_t** vals, unsigned long long* keys_alt,
                                 uint32_t* vals_alt, int64_t n, int nbits, uint32_t* temp, cudaStream_t s);
