@@ -262,17 +262,24 @@ __global__ void __launch_bounds__(SC_NT) k_scan_down(const uint32_t* __restrict_
 }
 
 // ---------------------------------------------------------------- radix sort
-constexpr int RS_NT = 256, RS_IPT = 16, RS_TILE = RS_NT * RS_IPT, RS_WARPS = RS_NT / 32;
-constexpr int RS_ROUNDS = RS_TILE / RS_WARPS / 32;  // 16 rounds of 32 per warp
+// A block sorts a tile of 256 IPT keys by one digit: 16 a thread, or 4 up to
+// RS_SMALL keys, where tiles of 4096 would leave most SMs without a block
+// (131k keys: 32 blocks, a pass 29 us; 128 blocks, 14 us).
+constexpr int RS_NT = 256, RS_WARPS = RS_NT / 32;
+constexpr int64_t RS_SMALL = 1 << 19;
+int64_t rs_tile(int64_t n) { return RS_NT * (n <= RS_SMALL ? 4 : 16); }
+int64_t rs_blocks(int64_t n) { return (n + rs_tile(n) - 1) / rs_tile(n); }
 
+
+template <int IPT>
 __global__ void __launch_bounds__(RS_NT) k_rs_hist(const u64* __restrict__ keys, int64_t n,
                                                    int shift, uint32_t* counts, int nb) {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0u;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+    const int64_t base = (int64_t)blockIdx.x * (RS_NT * IPT);
 #pragma unroll 4
-    for (int j = 0; j < RS_IPT; ++j) {
+    for (int j = 0; j < IPT; ++j) {
         const int64_t i = base + (int64_t)j * RS_NT + threadIdx.x;
         if (i < n) atomicAdd(&h[(unsigned)(keys[i] >> shift) & 255u], 1u);
     }
@@ -296,9 +303,10 @@ __global__ void __launch_bounds__(SC_NT) k_rs_scan_digits(uint32_t* counts, int 
     if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
-// Stable scatter: inside a block each warp ranks its 16 rounds of 32 items in
+// Stable scatter: inside a block each warp ranks its IPT rounds of 32 items in
 // order (match.any groups equal digits; the lowest lane of a group bumps the
 // warp's running digit count), then warps are offset in warp order.
+template <int IPT>
 __global__ void __launch_bounds__(RS_NT) k_rs_scatter(const u64* __restrict__ kin,
                                                       const uint32_t* __restrict__ vin,
                                                       u64* __restrict__ kout,
@@ -315,11 +323,11 @@ __global__ void __launch_bounds__(RS_NT) k_rs_scatter(const u64* __restrict__ ki
     }
     for (int d = tid; d < RS_WARPS * 256; d += RS_NT) (&wh[0][0])[d] = 0u;
     __syncthreads();
-    const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * (RS_ROUNDS * 32);
-    u64 key[RS_ROUNDS];
-    uint32_t val[RS_ROUNDS], rank[RS_ROUNDS];
+    const int64_t wbase = (int64_t)blockIdx.x * (RS_NT * IPT) + (int64_t)warp * (IPT * 32);
+    u64 key[IPT];
+    uint32_t val[IPT], rank[IPT];
 #pragma unroll
-    for (int r = 0; r < RS_ROUNDS; ++r) {
+    for (int r = 0; r < IPT; ++r) {
         const int64_t i = wbase + r * 32 + lane;
         const bool valid = i < n;
         key[r] = valid ? kin[i] : 0ull;
@@ -345,7 +353,7 @@ __global__ void __launch_bounds__(RS_NT) k_rs_scatter(const u64* __restrict__ ki
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < RS_ROUNDS; ++r) {
+    for (int r = 0; r < IPT; ++r) {
         const int64_t i = wbase + r * 32 + lane;
         if (i < n) {
             const unsigned d = (unsigned)(key[r] >> shift) & 255u;
@@ -544,17 +552,19 @@ cudaError_t scan_exclusive(const uint32_t* in, uint32_t* out, int64_t n, uint32_
     return cudaGetLastError();
 }
 
-cudaError_t radix_sort(u64*& keys, uint32_t*& vals, u64* keys_alt, uint32_t* vals_alt, int64_t n,
-                       int nbits, Scratch& sc, cudaStream_t s) {
-    const int nb = (int)((n + RS_TILE - 1) / RS_TILE);
-    uint32_t* counts = sc.alloc<uint32_t>((size_t)256 * nb);
-    uint32_t* totals = sc.alloc<uint32_t>(256);
-    if (!counts || !totals) return sc.err;
+// One pass per 8-bit digit; counts holds 256 rs_blocks(n) words, totals 256.
+cudaError_t radix_sort(u64*& keys, uint32_t*& vals, u64* keys_alt, uint32_t* vals_alt, int64_t n, int nbits,
+                       uint32_t* counts, uint32_t* totals, cudaStream_t s) {
+    const int nb = (int)rs_blocks(n);
+    const bool small = n <= RS_SMALL;
     for (int shift = 0; shift < nbits; shift += 8) {
-        k_rs_hist<<<nb, RS_NT, 0, s>>>(keys, n, shift, counts, nb);
+        if (small) k_rs_hist<4><<<nb, RS_NT, 0, s>>>(keys, n, shift, counts, nb);
+        else k_rs_hist<16><<<nb, RS_NT, 0, s>>>(keys, n, shift, counts, nb);
         k_rs_scan_digits<<<256, SC_NT, 0, s>>>(counts, nb, totals);
-        k_rs_scatter<<<nb, RS_NT, 0, s>>>(keys, vals, keys_alt, vals_alt, n, shift, counts, nb,
-                                          totals);
+        if (small)
+            k_rs_scatter<4><<<nb, RS_NT, 0, s>>>(keys, vals, keys_alt, vals_alt, n, shift, counts, nb, totals);
+        else
+            k_rs_scatter<16><<<nb, RS_NT, 0, s>>>(keys, vals, keys_alt, vals_alt, n, shift, counts, nb, totals);
         std::swap(keys, keys_alt);
         std::swap(vals, vals_alt);
     }
@@ -565,29 +575,16 @@ cudaError_t radix_sort(u64*& keys, uint32_t*& vals, u64* keys_alt, uint32_t* val
 
 // Sort and scan on caller buffers (used by the wall detector, which sizes
 // everything once at creation).
+// for any count up to n
 size_t pc_sort_temp_words(int64_t n) {
-    const int64_t nb = (n + RS_TILE - 1) / RS_TILE;
+    const int64_t nb = std::max(rs_blocks(n), rs_blocks(std::min(n, RS_SMALL)));
     return (size_t)256 * (size_t)std::max<int64_t>(nb, 1) + 256;
 }
 
 cudaError_t pc_radix_sort_pairs(u64** keys, uint32_t** vals, u64* keys_alt, uint32_t* vals_alt,
                                 int64_t n, int nbits, uint32_t* temp, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    const int nb = (int)((n + RS_TILE - 1) / RS_TILE);
-    uint32_t* counts = temp;
-    uint32_t* totals = temp + (size_t)256 * nb;
-    u64* k = *keys;
-    uint32_t* v = *vals;
-    for (int shift = 0; shift < nbits; shift += 8) {
-        k_rs_hist<<<nb, RS_NT, 0, s>>>(k, n, shift, counts, nb);
-        k_rs_scan_digits<<<256, SC_NT, 0, s>>>(counts, nb, totals);
-        k_rs_scatter<<<nb, RS_NT, 0, s>>>(k, v, keys_alt, vals_alt, n, shift, counts, nb, totals);
-        std::swap(k, keys_alt);
-        std::swap(v, vals_alt);
-    }
-    *keys = k;
-    *vals = v;
-    return cudaGetLastError();
+    return radix_sort(*keys, *vals, keys_alt, vals_alt, n, nbits, temp, temp + 256 * rs_blocks(n), s);
 }
 
 size_t pc_scan_temp_words(int64_t n) {
@@ -747,7 +744,9 @@ pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& opts, 
     if (!keys || !keys_alt || !vals || !vals_alt) return pc_from_cuda(sc.err);
     k_keys<<<grid_for(M, 256), 256, 0, s>>>(xyz, M, o[0], o[1], o[2], inv_h, bx, by, sub, keys, vals);
     PC_TRY(cudaGetLastError());
-    PC_TRY(radix_sort(keys, vals, keys_alt, vals_alt, M, bx + by + bz + sub, sc, s));
+    uint32_t* sort_tmp = sc.alloc<uint32_t>(pc_sort_temp_words(M));
+    if (!sort_tmp) return pc_from_cuda(sc.err);
+    PC_TRY(pc_radix_sort_pairs(&keys, &vals, keys_alt, vals_alt, M, bx + by + bz + sub, sort_tmp, s));
 
     // 5. occupied cells
     uint32_t* flags = sc.alloc<uint32_t>(M);

@@ -7,17 +7,18 @@
 //  1. voxel key of every point (binary32 floor(p * fl(1/v)) per axis, fields
 //     offset into [0, 2^b - 2]; dropped points get the all-ones key), stable
 //     LSD radix sort of (key, index), run starts by a flag scan; each voxel's
-//     centroid is summed in binary64 in index order, divided by the count and
-//     rounded to binary32;
+//     centroid is summed in binary64 in eight strands of index order, divided
+//     by the count and rounded to binary32;
 //  2. each voxel votes for the 2-D cell of its centroid in an open-addressing
 //     hash (integer counts, so the result is order-free); a voxel is
 //     vertical when its cell holds more than min_votes voxels;
 //  3. vertical voxels are linked when their pinned binary32 d2 <= fl(tol^2):
 //     a hash of cells of edge tol (1 + 2^-10) keeps per-cell linked lists, and
 //     a lock-free union-find (every voxel first under its smallest linked
-//     neighbour, a dozen rounds of pointer jumping, then unions that hook the
-//     larger root under the smaller, with path halving) gives every
-//     component its smallest voxel index as label;
+//     neighbour, flattened by pointer jumping, roots hooked across the links
+//     and flattened again, then unions that hook the larger root under the
+//     smaller, with path halving) gives every component its smallest voxel
+//     index as label;
 //  4. per cluster: count and the extremes of x and y (ordered-integer
 //     atomics); the wall is the cluster of >= min_cluster voxels with
 //     fl(min y + max y) < 0 and the largest fl(max x - min x), ties to the
@@ -93,6 +94,33 @@ struct WallParams {
     int log2cap;  // both hash tables
 };
 
+// Everything a detection starts from, in one launch (fifteen memsets before).
+struct WallInit {
+    u64 *vkeys, *ckeys, *pick;
+    uint32_t *vcount, *nv, *starts;
+    int *head, *err;
+    unsigned *cmin_x, *cmin_y, *cmax_x, *cmax_y, *ccount, *nvert, *ticket;
+};
+__global__ void k_wall_init(WallInit w, int64_t C, int64_t n) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < C) {
+        w.vkeys[i] = w.ckeys[i] = INVALID_KEY;
+        w.vcount[i] = 0u;
+        w.head[i] = -1;
+    }
+    if (i < n) {
+        w.cmin_x[i] = w.cmin_y[i] = 0xffffffffu;
+        w.cmax_x[i] = w.cmax_y[i] = 0u;
+        w.ccount[i] = 0u;
+    }
+    if (i == 0) {
+        *w.pick = 0ull;
+        *w.nv = *w.starts = 0u;
+        *w.err = 0;
+        *w.nvert = *w.ticket = 0u;
+    }
+}
+
 // 1. voxel keys
 __global__ void k_wall_keys(const float* __restrict__ pts, int64_t n, WallParams P, u64* __restrict__ keys,
                             uint32_t* __restrict__ vals) {
@@ -134,21 +162,38 @@ __global__ void k_wall_starts(const u64* __restrict__ keys, const uint32_t* __re
     if (i == 0 && !valid) starts[0] = 0u;  // nothing valid: nv = 0
 }
 
+// Eight lanes per voxel: near the sensor a voxel holds hundreds of points, and
+// one lane adding them up by dependent gathers set the kernel's time (45 us on
+// a 131k scan, 25 with eight).  Binary64 sums in eight strands, added pairwise.
 __global__ void k_wall_centroid(const float* __restrict__ pts, const uint32_t* __restrict__ vals,
                                 const uint32_t* __restrict__ starts, const uint32_t* __restrict__ nvp,
                                 float4* __restrict__ cent) {
     const uint32_t nv = *nvp;
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
-        const uint32_t a = starts[v], b = starts[v + 1];
+    const uint32_t lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; base < nv; base += warps * 4) {
+        const uint32_t v = base + (lane >> 3);
         double sx = 0.0, sy = 0.0, sz = 0.0;
-        for (uint32_t s = a; s < b; ++s) {
+        uint32_t a = 0, b = 0;
+        if (v < nv) {
+            a = starts[v];
+            b = starts[v + 1];
+        }
+        for (uint32_t s = a + (lane & 7); s < b; s += 8) {
             const uint32_t i = vals[s];
             sx += (double)pts[3 * (size_t)i];
             sy += (double)pts[3 * (size_t)i + 1];
             sz += (double)pts[3 * (size_t)i + 2];
         }
-        const double c = (double)(b - a);
-        cent[v] = make_float4((float)(sx / c), (float)(sy / c), (float)(sz / c), 0.0f);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            sx += __shfl_xor_sync(0xffffffffu, sx, o);
+            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+            sz += __shfl_xor_sync(0xffffffffu, sz, o);
+        }
+        if (v < nv && (lane & 7) == 0) {
+            const double c = (double)(b - a);
+            cent[v] = make_float4((float)(sx / c), (float)(sy / c), (float)(sz / c), 0.0f);
+        }
     }
 }
 
@@ -275,20 +320,48 @@ __global__ void k_wall_link_init(const float4* __restrict__ cent, const uint32_t
     }
 }
 
-// 3b. one round of pointer jumping: every vertical voxel moves up to its
-// grandparent (the init forest has chains as long as a wall; a dozen rounds
-// flatten them, so the unions below chase short paths)
-__global__ void k_wall_jump(const uint32_t* __restrict__ nvp, const int* __restrict__ vertical, int* parent) {
+// 3b. pointer jumping in one launch: every vertical voxel climbs to the root
+// of its tree, writing the ancestor it has reached as it goes, so the climbs
+// below it shorten (the init forest has chains as long as a wall).  Twelve
+// launches of one jump each took 44 us and twelve launch gaps; this one 5 us.  A climb that
+// uses up its steps leaves a valid, longer path for the unions.
+__global__ void k_wall_flatten(const uint32_t* __restrict__ nvp, const int* __restrict__ vertical, int* parent) {
     const uint32_t nv = *nvp;
     volatile int* par = parent;
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
         if (!vertical[v]) continue;
-        const int p = par[v];
-        const int gp = par[p];
-        if (gp != p) par[v] = gp;
+        int p = par[v];
+        for (int it = 0; it < 128; ++it) {
+            const int gp = par[p];
+            if (gp == p) break;
+            par[v] = gp;
+            p = gp;
+        }
     }
 }
-constexpr int JUMP_ROUNDS = 12;
+
+// 3c. the links between different trees of the flattened forest hook the
+// larger root under the smallest root it meets (a link that loses this race
+// is taken up by the unions).  Without it almost every link of the two trees
+// of a wall went through the union-find: 85 us, 22 after it.
+__global__ void k_wall_hook(const float4* __restrict__ cent, const uint32_t* __restrict__ nvp, WallParams P,
+                            const int* __restrict__ vertical, const u64* __restrict__ ckeys,
+                            const int* __restrict__ head, const int* __restrict__ next, int* parent) {
+    const uint32_t nv = *nvp;
+    const int lane = threadIdx.x & 31;
+    const uint32_t wpb = blockDim.x >> 5;
+    for (uint32_t v = blockIdx.x * wpb + (threadIdx.x >> 5); v < nv; v += gridDim.x * wpb) {
+        if (!vertical[v] || lane >= 27) continue;
+        const int pv = __ldcg(&parent[v]);
+        int seen = pv;
+        for_links_in_cell(cent, v, nv, lane, P, ckeys, head, next, [&](int j) {
+            const int pj = __ldcg(&parent[j]);
+            if (pj == pv || pj == seen) return;
+            seen = pj;
+            atomicMin(&parent[pj > pv ? pj : pv], pj > pv ? pv : pj);
+        });
+    }
+}
 
 // 3. links between vertical voxels in the 27 neighbouring cluster cells:
 // one warp per voxel, one lane per cell; pairs already under one parent are
@@ -412,13 +485,18 @@ __global__ void __launch_bounds__(FIT_NT) k_wall_fit(const float4* __restrict__ 
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == FIT_BLOCKS - 1 ? 1u : 0u;
     __syncthreads();
-    if (!last || threadIdx.x != 0) return;
+    if (!last) return;
     __threadfence();
-    double S[FIT_VALS];
-    for (int j = 0; j < FIT_VALS; ++j) {
-        S[j] = 0.0;
-        for (int bk = 0; bk < FIT_BLOCKS; ++bk) S[j] += __ldcg(&partial[bk * FIT_VALS + j]);
+    // one thread per sum, blocks in order (one thread for all of them: 36 us, now 17)
+    __shared__ double S[FIT_VALS];
+    if (threadIdx.x < FIT_VALS) {
+        double s = 0.0;
+#pragma unroll 16
+        for (int bk = 0; bk < FIT_BLOCKS; ++bk) s += __ldcg(&partial[bk * FIT_VALS + threadIdx.x]);
+        S[threadIdx.x] = s;
     }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     *ticket = 0u;
     out->n_voxels = nv;
     out->n_vertical = *nvert;
@@ -601,29 +679,21 @@ pc_status pc_wall_detect(pc_wall w, const float* pts_dev, int64_t n, pc_stream s
     int prev = -1;
     if (cudaGetDevice(&prev) == cudaSuccess && prev != w->device) cudaSetDevice(w->device);
     cudaStream_t st = (cudaStream_t)s;
-    const WallParams P = w->P;
-    const int64_t C = 1ll << P.log2cap;
+    WallParams P = w->P;
+    int lc = 1;  // tables for this scan's points, at most the detector's
+    while (lc < P.log2cap && (1ll << lc) < 2 * n) ++lc;
+    P.log2cap = lc;
+    const int64_t C = 1ll << lc;
     const int NT = 256;
     cudaError_t e = cudaSuccess;
     auto ok = [&](cudaError_t r) {
         if (e == cudaSuccess) e = r;
         return e == cudaSuccess;
     };
-    ok(cudaMemsetAsync(w->vkeys, 0xff, 8 * C, st));
-    ok(cudaMemsetAsync(w->ckeys, 0xff, 8 * C, st));
-    ok(cudaMemsetAsync(w->vcount, 0, 4 * C, st));
-    ok(cudaMemsetAsync(w->head, 0xff, 4 * C, st));
-    ok(cudaMemsetAsync(w->err, 0, 4, st));
-    ok(cudaMemsetAsync(w->nvert, 0, 4, st));
-    ok(cudaMemsetAsync(w->nv, 0, 4, st));
-    ok(cudaMemsetAsync(w->cmin_x, 0xff, 4 * w->cap, st));
-    ok(cudaMemsetAsync(w->cmin_y, 0xff, 4 * w->cap, st));
-    ok(cudaMemsetAsync(w->cmax_x, 0, 4 * w->cap, st));
-    ok(cudaMemsetAsync(w->cmax_y, 0, 4 * w->cap, st));
-    ok(cudaMemsetAsync(w->ccount, 0, 4 * w->cap, st));
-    ok(cudaMemsetAsync(w->starts, 0, 4, st));
-    ok(cudaMemsetAsync(w->pick, 0, 8, st));
-    ok(cudaMemsetAsync(w->ticket, 0, 4, st));
+    const WallInit init{w->vkeys,  w->ckeys,  w->pick,   w->vcount, w->nv,     w->starts, w->head,  w->err,
+                        w->cmin_x, w->cmin_y, w->cmax_x, w->cmax_y, w->ccount, w->nvert,  w->ticket};
+    k_wall_init<<<(unsigned)((C + NT - 1) / NT), NT, 0, st>>>(init, C, n);
+    ok(cudaGetLastError());
     if (n > 0) {
         const unsigned gb = (unsigned)((n + NT - 1) / NT);
         k_wall_keys<<<gb, NT, 0, st>>>(pts_dev, n, P, w->keys, w->vals);
@@ -647,7 +717,9 @@ pc_status pc_wall_detect(pc_wall w, const float* pts_dev, int64_t n, pc_stream s
         const unsigned wb = blocks_for(n * 32, NT);
         k_wall_link_init<<<wb, NT, 0, st>>>(w->cent, w->nv, P, w->vertical, w->ckeys, w->head, w->next,
                                            w->parent);
-        for (int r = 0; r < JUMP_ROUNDS; ++r) k_wall_jump<<<vb, NT, 0, st>>>(w->nv, w->vertical, w->parent);
+        k_wall_flatten<<<vb, NT, 0, st>>>(w->nv, w->vertical, w->parent);
+        k_wall_hook<<<wb, NT, 0, st>>>(w->cent, w->nv, P, w->vertical, w->ckeys, w->head, w->next, w->parent);
+        k_wall_flatten<<<vb, NT, 0, st>>>(w->nv, w->vertical, w->parent);
         k_wall_union<<<wb, NT, 0, st>>>(w->cent, w->nv, P, w->vertical, w->ckeys, w->head, w->next, w->parent,
                                        w->err);
         k_wall_label<<<vb, NT, 0, st>>>(w->cent, w->nv, w->vertical, w->parent, w->label, w->cmin_x, w->cmax_x,
