@@ -516,20 +516,23 @@ __global__ void __launch_bounds__(512) k_rho_hints(const float* __restrict__ d2,
 }
 
 // ---------------------------------------------------------------- host helpers
+// The build's temporaries, given back in the order of its stream.
 struct Scratch {
+    cudaStream_t s;
     std::vector<void*> bufs;
     cudaError_t err = cudaSuccess;
+    explicit Scratch(cudaStream_t st) : s(st) {}
     template <typename T>
     T* alloc(size_t count) {
         void* p = nullptr;
         if (err != cudaSuccess) return nullptr;
-        err = cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(T));
+        err = pc_dev_alloc(&p, std::max<size_t>(count, 1) * sizeof(T), s);
         if (err != cudaSuccess) return nullptr;
         bufs.push_back(p);
         return static_cast<T*>(p);
     }
     ~Scratch() {
-        for (void* p : bufs) cudaFree(p);
+        for (void* p : bufs) pc_dev_free(p, s);
     }
 };
 
@@ -644,10 +647,9 @@ cudaError_t pc_launch_rho_hints(const float* d2, int n, int kc, float* out, cuda
 }
 
 void pc_free_grid(pc_target_s* t) {
-    void* ps[] = {t->table, t->pts, t->xyz, t->cell_keys, t->cell_start, t->status, t->stage,
-                  t->dstart, t->xcut};
-    for (void* p : ps)
-        if (p) cudaFree(p);
+    void* const ps[] = {t->table, t->pts, t->xyz, t->cell_keys, t->cell_start, t->status, t->dstart, t->xcut};
+    pc_dev_free_idle(ps, 8);
+    if (t->stage) cudaFree(t->stage);
     t->table = nullptr;
     t->pts = t->xyz = nullptr;
     t->cell_keys = nullptr;
@@ -667,10 +669,11 @@ void pc_free_grid(pc_target_s* t) {
 
 pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& opts, cudaStream_t s,
                         pc_target_s* t) {
-    Scratch sc;
+    Scratch sc(s);
+    auto keep = [&](auto** p, size_t bytes) { return pc_dev_alloc(reinterpret_cast<void**>(p), bytes, s); };
     // persistent small buffers first
     // status word + statistics counters (64 bytes)
-    PC_TRY(cudaMalloc(&t->status, 64));
+    PC_TRY(keep(&t->status, 64));
     PC_TRY(cudaMemsetAsync(t->status, 0, 64, s));
 
     // 1. bbox + finite check
@@ -758,8 +761,8 @@ pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& opts, 
     uint32_t U = 0;
     PC_TRY(cudaMemcpyAsync(&U, total_dev, sizeof(U), cudaMemcpyDeviceToHost, s));
     PC_TRY(cudaStreamSynchronize(s));
-    PC_TRY(cudaMalloc(&t->cell_keys, sizeof(u64) * std::max<uint32_t>(U, 1)));
-    PC_TRY(cudaMalloc(&t->cell_start, sizeof(uint32_t) * ((size_t)U + 1)));
+    PC_TRY(keep(&t->cell_keys, sizeof(u64) * std::max<uint32_t>(U, 1)));
+    PC_TRY(keep(&t->cell_start, sizeof(uint32_t) * ((size_t)U + 1)));
     k_cells<<<grid_for(M, 256), 256, 0, s>>>(keys, flags, ord, M, sub, t->cell_keys, t->cell_start, U);
     PC_TRY(cudaGetLastError());
 
@@ -768,7 +771,7 @@ pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& opts, 
     int log2cap = 1;
     while ((double)(1ll << log2cap) * load < (double)U) ++log2cap;
     t->table_cap = 1ll << log2cap;
-    PC_TRY(cudaMalloc(&t->table, sizeof(uint4) * (size_t)t->table_cap));
+    PC_TRY(keep(&t->table, sizeof(uint4) * (size_t)t->table_cap));
     PC_TRY(cudaMemsetAsync(t->table, 0xff, sizeof(uint4) * (size_t)t->table_cap, s));
     k_hash_insert<<<grid_for(U, 256), 256, 0, s>>>(t->cell_keys, t->cell_start, U, t->table,
                                                     log2cap);
@@ -789,12 +792,12 @@ pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& opts, 
         k_popc<<<grid_for(nwords, 256), 256, 0, s>>>(occ, nwords, pop);
         PC_TRY(cudaGetLastError());
         PC_TRY(scan_exclusive(pop, rank, nwords, tot2, sc, s));
-        PC_TRY(cudaMalloc(&t->dstart, sizeof(uint32_t) * (size_t)(ngrid + 1)));
+        PC_TRY(keep(&t->dstart, sizeof(uint32_t) * (size_t)(ngrid + 1)));
         k_dstart<<<grid_for(ngrid + 1, 256), 256, 0, s>>>(occ, rank, t->cell_start, ngrid, U, t->dstart);
         PC_TRY(cudaGetLastError());
         dense_words = ngrid + 1;
         if (sub) {  // 6c. sub-cell cut
-            PC_TRY(cudaMalloc(&t->xcut, sizeof(uint2) * (size_t)ngrid));
+            PC_TRY(keep(&t->xcut, sizeof(uint2) * (size_t)ngrid));
             PC_TRY(cudaMemsetAsync(t->xcut, 0, sizeof(uint2) * (size_t)ngrid, s));
             k_xcut<<<grid_for(M, 256), 256, 0, s>>>(keys, M, bx, by, dims[0], dims[1], t->dstart,
                                                       reinterpret_cast<unsigned char*>(t->xcut));
@@ -804,8 +807,8 @@ pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& opts, 
     }
 
     // 7. float4 copies
-    PC_TRY(cudaMalloc(&t->pts, sizeof(float4) * (size_t)M));
-    PC_TRY(cudaMalloc(&t->xyz, sizeof(float4) * (size_t)M));
+    PC_TRY(keep(&t->pts, sizeof(float4) * (size_t)M));
+    PC_TRY(keep(&t->xyz, sizeof(float4) * (size_t)M));
     k_gather<<<grid_for(M, 256), 256, 0, s>>>(xyz, vals, M, t->pts, t->xyz);
     PC_TRY(cudaGetLastError());
     PC_TRY(cudaStreamSynchronize(s));

@@ -1,0 +1,78 @@
+// Device memory of targets and of their builds, from one stream-ordered pool
+// per device.  A build makes about 25 allocations; through cudaMalloc and
+// cudaFree each took 40-90 us (and every cudaFree waited for the device): with them
+// a 131k-point target took 1.19 ms to build and 0.25 ms to close, with the pool
+// 0.55 and 0.01.  The pool keeps at most POOL_KEEP bytes when
+// nothing uses them and gives the rest back to the device at the next
+// synchronisation; an allocation that finds no memory first gives back all of
+// it and tries again.  The pool's own calls are safe from any thread.
+#include <mutex>
+
+#include "pc_internal.h"
+
+namespace {
+
+constexpr uint64_t POOL_KEEP = 256ull << 20;
+
+struct Pool {
+    bool made;
+    cudaMemPool_t pool;   // null: the device has no pools (plain allocations then)
+    cudaStream_t frees;   // memory whose last use is known to be over is freed here
+};
+std::mutex g_pool_mu;
+Pool g_pools[64];
+
+Pool* current_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    Pool& p = g_pools[dev];
+    if (p.made) return &p;
+    p.made = true;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = POOL_KEEP;
+    if (cudaStreamCreateWithFlags(&p.frees, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaMemPoolCreate(&p.pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        p.pool = nullptr;
+    }
+    return &p;
+}
+
+}  // namespace
+
+cudaError_t pc_dev_alloc(void** out, size_t bytes, cudaStream_t s) {
+    Pool* p = current_pool();
+    if (!p) return cudaErrorInvalidDevice;
+    if (!p->pool) return cudaMalloc(out, bytes);
+    cudaError_t e = cudaMallocFromPoolAsync(out, bytes, p->pool, s);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        cudaStreamSynchronize(s);
+        cudaMemPoolTrimTo(p->pool, 0);
+        e = cudaMallocFromPoolAsync(out, bytes, p->pool, s);
+    }
+    return e;
+}
+
+void pc_dev_free(void* ptr, cudaStream_t s) {
+    Pool* p = current_pool();
+    if (!ptr || !p) return;
+    if (p->pool) cudaFreeAsync(ptr, s);
+    else cudaFree(ptr);
+}
+
+void pc_dev_free_idle(void* const* ptrs, int n) {
+    Pool* p = current_pool();
+    if (!p) return;
+    if (p->pool) cudaDeviceSynchronize();  // as cudaFree does: the caller's streams may still use them
+    for (int i = 0; i < n; ++i) {
+        if (!ptrs[i]) continue;
+        if (p->pool) cudaFreeAsync(ptrs[i], p->frees);
+        else cudaFree(ptrs[i]);
+    }
+}

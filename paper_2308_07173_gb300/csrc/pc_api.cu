@@ -98,7 +98,7 @@ pc_status calibrate_rho(pc_target_s* t, cudaStream_t s) {
     const int64_t S = std::min<int64_t>(M, 1024);
     float* buf = nullptr;  // sample points, distances, hints, indices
     const size_t words = (size_t)S * 3 + (size_t)S * kc * 2 + 66;
-    cudaError_t e = cudaMalloc(&buf, words * sizeof(float));
+    cudaError_t e = pc_dev_alloc(reinterpret_cast<void**>(&buf), words * sizeof(float), s);
     if (e != cudaSuccess) return pc_from_cuda(e);
     float* const q = buf;
     float* const d2 = q + 3 * S;
@@ -112,7 +112,7 @@ pc_status calibrate_rho(pc_target_s* t, cudaStream_t s) {
     // the status word and statistics start clean (a capped search here only skips that sample)
     if (e == cudaSuccess) e = cudaMemsetAsync(t->status, 0, 64, s);
     const cudaError_t e2 = cudaStreamSynchronize(s);
-    cudaFree(buf);
+    pc_dev_free(buf, s);
     if (e != cudaSuccess || e2 != cudaSuccess) return pc_from_cuda(e != cudaSuccess ? e : e2);
     std::memcpy(t->rho_hint, h, 64 * sizeof(float));
     // spread of the distances at k = min(kc, 16): a map whose density varies
@@ -147,6 +147,12 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 // searched with one trial radius, and an append costs one grid build.
 static pc_status build_target_internal(const float* xyz, int64_t M, const pc_build_opts& o, cudaStream_t st,
                                        pc_target_s** out, const pc_target_s* like = nullptr) {
+    // a build cannot be captured: refuse before anything is queued or allocated
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return PC_ERR_CUDA;
+    }
     pc_target_s* t = new (std::nothrow) pc_target_s();
     if (!t) return PC_ERR_OOM;
     std::memset(t, 0, sizeof(*t));

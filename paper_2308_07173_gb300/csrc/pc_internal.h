@@ -110,6 +110,13 @@ inline void pc_clear_window(pcdev::Grid& g) {
     g.whix = g.whiy = g.whiz = INFINITY;
 }
 
+// mem.cu: device memory of targets on the current device, ready for use in
+// the order of stream s.  pc_dev_free: after the work queued on s;
+// pc_dev_free_idle: after a device synchronisation, for any stream's users.
+cudaError_t pc_dev_alloc(void** out, size_t bytes, cudaStream_t s);
+void pc_dev_free(void* ptr, cudaStream_t s);
+void pc_dev_free_idle(void* const* ptrs, int n);
+
 // grid_build.cu
 pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& o, cudaStream_t s,
                         pc_target_s* t);
