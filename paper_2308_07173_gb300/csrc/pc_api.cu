@@ -833,14 +833,15 @@ pc_status pc_gicp_linearize(pc_target map, const float* map_cov_dev, const float
     const size_t need = pc_gicp_work_size();
     if (need == 0) return PC_ERR_CUDA;
     if (work_bytes < need) return PC_ERR_INVALID_ARG;
-    // start radius: the calibrated distance to the nearest other map point
-    float r0 = pc_rho0(map, map->g.m >= 2 ? 2 : 1);
-    if (!(r0 > 0.0f)) r0 = map->g.h;
-    float r0d = r0;
-    if (map->delta) {
-        r0d = pc_rho0(map->delta, map->delta->g.m >= 2 ? 2 : 1);
-        if (!(r0d > 0.0f)) r0d = map->delta->g.h;
-    }
+    // Start radius: the calibrated distance to a map point's 8th neighbour
+    // (itself included).  A shorter one makes most warps search twice, a longer
+    // one visits more points: 100k points against 2M, ten iterations, with the
+    // 2nd, 4th, 8th, 16th: 697, 640, 615, 755 us.
+    auto start = [](const pc_target_s* t) {
+        const float r = pc_rho0(t, (int)std::min<int64_t>(t->g.m, 8));
+        return r > 0.0f ? r : t->g.h;
+    };
+    const float r0 = start(map), r0d = map->delta ? start(map->delta) : r0;
     return pc_from_cuda(pc_launch_gicp_linearize(map, map_cov_dev, src_dev, n, src_cov_dev, pose_dev,
                                                  max_dist, out_dev, corr_dev, work_dev, r0, r0d,
                                                  (cudaStream_t)s));
