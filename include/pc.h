@@ -75,27 +75,28 @@ typedef struct {
                           mean points per occupied cell is about `occupancy` */
     float occupancy;   /* target mean points per occupied cell for the automatic h; <= 0: 12 */
     float hash_load;   /* open-addressing load factor in (0, 0.9]; <= 0: 0.5 */
-    int max_box_cells; /* the radius-widening search stops growing its cell box here; <= 0: 4096 */
-    int exhaustive;    /* past max_box_cells: 1 = exact scan of every occupied cell,
+    int max_box_cells; /* the radius-widening search stops growing its cell box here; <= 0: 4096
+                          (with exhaustive = 1 and a row index kNN searches go on by rows) */
+    int exhaustive;    /* past that: 1 = exact scan of every occupied cell,
                           0 = mark the row and report PC_ERR_SEARCH_LIMIT */
 } pc_build_opts;
 
 /* Launch shape of the search kernel.  None of these changes any result. */
 typedef struct {
-    int tile;          /* queries per warp work item (one per lane for k <= 32), 1..32;
-                          <= 0: 32 */
-    int warps;         /* warps per block, 1..8; <= 0: 4 */
+    int tile;          /* k > 32: most queries per warp work item, 1..32; <= 0: 32 (k <= 32
+                          searches run units of 4 or 8 queries by the call's size) */
+    int warps;         /* k > 32: warps per block, 1..8; <= 0: 4 */
     float rho_scale;   /* scales the target's calibrated k-th-neighbour radius that the
-                          search starts from (k <= 32: trial radii 0.75..1.46 x it);
+                          search starts from (k <= 32: at 1.4 x it);
                           <= 0: 0.9 */
     int order;         /* 0: issue query tiles last-first (a ring-by-ring LiDAR scan ends
                           with its slowest, farthest rings); 1: first-first */
-    int probe;         /* where each query's trial radii start (k <= 32): 0 auto (1 on a
+    int probe;         /* where each query's radius starts (k <= 32): 0 auto (1 on a
                           map whose calibration saw an even density, else 2); 1 the
                           calibrated radius for every query; 2 a per-query radius from
                           the point count of the 27 cells around it */
-    int slots;         /* survivor slots per query of the lane path (its k tile): 0 by
-                          k (32 for k <= 24, 64 for 25..32); 64 for every k <= 32 */
+    int slots;         /* points per query that are sorted (k <= 32): 0 by k (32 for k <=
+                          24, 64 for 25..32); 64 for every k <= 32 */
 } pc_tune;
 
 /* What the built target looks like (for reporting and tuning). */
@@ -118,19 +119,17 @@ typedef struct {
 typedef struct {
     int64_t queries;     /* queries answered */
     int64_t warp_search; /* of those, answered by the warp-cooperative search
-                            (k > 32, or k <= 32 queries the lane path handed over) */
+                            (k > 32, or k <= 32 queries the group search handed over) */
     int64_t exhaustive;  /* searches that ended in the exhaustive cell scan */
-    int64_t candidates;  /* target points whose distance the lane path computed
-                            (its counting and collecting passes together) */
+    int64_t candidates;  /* target points whose distance the group search computed */
 } pc_stats;
 
 /* One scan of a batch, caller-owned: device memory, or page-locked host
  * memory mapped into the device's address space (cudaHostAlloc,
  * cudaHostRegister, torch pin_memory).  When any scan's idx, d2 or cov is
- * such host memory, the batch runs the staged kernel: each warp writes its
- * tile's rows as whole blocks, so the results reach host memory during the
- * search with no copy (for k <= 32; the warp path, k > 32, writes its rows
- * directly).  Results are identical either way.  Any other pointer returns
+ * such host memory, each warp writes its queries' rows as whole blocks, so
+ * the results reach host memory during the search with no copy (for k <= 32;
+ * the warp path, k > 32, writes row by row).  Results are identical either way.  Any other pointer returns
  * PC_ERR_BAD_POINTER. */
 typedef struct {
     const float *q_dev; /* [n,3] */

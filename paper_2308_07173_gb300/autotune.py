@@ -6,13 +6,11 @@ cell size, launch shape or starting radius), so the tuner only times them:
 * occupancy -- target mean points per occupied cell, which sets the cell
   edge h of the voxel-hash grid (the target is rebuilt per value);
 * rho_scale -- the starting radius as a multiple of the calibrated k-th
-  neighbour distance (the lane path's trial radii scale with it);
-* warps -- warps per block;
-* tile -- queries per warp work item (points per warp: 32 fills every lane
-  of the lane path, fewer leave lanes idle but shorten each item);
-* slots -- the lane path's survivor slots per query, its k tile: 32 (k <=
-  24) with eight trial radii, or 64 with four;
-* probe -- whether each query's trial radii start from the map's
+  neighbour distance (k <= 32 searches start at 1.4 x it);
+* warps -- warps per block (k > 32);
+* tile -- most queries per warp work item (k > 32);
+* slots -- points per query that are sorted (k <= 32): 32 (k <= 24) or 64;
+* probe -- whether each query's radius starts from the map's
   calibrated radius (1) or from a per-query estimate from the point count
   of the 27 cells around it (2).
 

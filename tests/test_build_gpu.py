@@ -49,3 +49,33 @@ def test_cell_size_and_hints(gpu_lib, m):
     want = np.zeros(64, F)
     want[:kc] = np.sqrt(np.sort(d2, axis=0)[s * 3 // 4])
     np.testing.assert_array_equal(np.array(i["rho_hint"], F), want)
+
+
+@pytest.mark.parametrize("m", [1024, 1025, 524288, 524289])
+def test_sort_tile_edges(gpu_lib, m):
+    """Both sort tiles and their remainders: every point is found where it is."""
+    p = (np.random.default_rng(m).random((m, 3)) * [300, 200, 3]).astype(F)
+    t = gpu_lib.Target(torch.from_numpy(p).cuda())
+    at = np.unique(np.concatenate([np.arange(0, m, max(1, m // 4000)), [m - 1]]))
+    idx, d2 = t.knn(torch.from_numpy(p[at]).cuda(), 1)
+    t.close()
+    assert (d2 == 0).all()
+    np.testing.assert_array_equal(p[idx.cpu().numpy()[:, 0]], p[at])
+
+
+@pytest.mark.parametrize("n", [1, 300, 5000, 70000])
+def test_wall_of_a_small_scan_in_a_large_detector(gpu_lib, n):
+    """A detector made for 600k points (its tables and sort follow the scan)."""
+    from paper_2308_07173_gb300 import workloads as W
+
+    pts = torch.from_numpy(np.ascontiguousarray(W.body_frame_scan(seed=3)[:n])).cuda()
+    got = []
+    for cap in (n, 600_000):
+        det = gpu_lib.WallDetector(cap)
+        det.detect(pts)
+        got.append(det.result(arrays=True))
+        det.close()
+    a, b = got
+    assert a.keys() == b.keys()
+    for k in a:
+        np.testing.assert_array_equal(np.asarray(a[k]), np.asarray(b[k]))
