@@ -146,7 +146,8 @@ PC_API void pc_default_build_opts(pc_build_opts *o);
  * (Sec. III-C3 "GPU-hash data structure"): finite check and bounding box,
  * cell keys, an LSD radix sort of (key, index), the occupied-cell table in an
  * open-addressing hash, and cell-ordered float4 copies of the points.  The
- * library copies the points; xyz_dev may be freed afterwards.  Synchronises
+ * library copies the points; xyz_dev may be freed afterwards.  Memory comes from
+ * a pool of the library that keeps up to 256 MB per device for later targets.  Synchronises
  * `s` (it reads sizes back).  opts may be NULL (defaults).  Errors:
  * PC_ERR_INVALID_ARG (M < 1 or M >= 2^31, NULL pointers), PC_ERR_BAD_POINTER,
  * PC_ERR_NONFINITE (any NaN/inf coordinate; no handle is made), PC_ERR_OOM,

@@ -605,7 +605,7 @@ __device__ void cov_row_union(const Grid& g, const Grid& dg, const int32_t* nb, 
 //   w_j = K(x, y_j),  W = sum w_j,
 //   mu = sum w_j y_j / W,  C = sum w_j (y_j - mu)(y_j - mu)^T / W,
 // then, for eps >= 0, C' = I - (1 - eps) n n^T with n the smallest-eigenvalue
-// eigenvector (the same Jacobi solver as the plain covariance).  Binary32,
+// eigenvector (the same closed form as the plain covariance).  Binary32,
 // two passes shifted by the nearest neighbour y_0 like the plain form.  A row
 // whose W is not positive and finite is NaN.  The search kernels call it in
 // place of cov_core when a descriptor is set, reading the neighbours from the

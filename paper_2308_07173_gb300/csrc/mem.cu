@@ -69,7 +69,13 @@ void pc_dev_free(void* ptr, cudaStream_t s) {
 void pc_dev_free_idle(void* const* ptrs, int n) {
     Pool* p = current_pool();
     if (!p) return;
-    if (p->pool) cudaDeviceSynchronize();  // as cudaFree does: the caller's streams may still use them
+    // as cudaFree does: the caller's streams may still use them.  Where that is
+    // refused (this thread is capturing), the memory stays allocated, as it did
+    // when cudaFree was refused.
+    if (p->pool && cudaDeviceSynchronize() != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
     for (int i = 0; i < n; ++i) {
         if (!ptrs[i]) continue;
         if (p->pool) cudaFreeAsync(ptrs[i], p->frees);
