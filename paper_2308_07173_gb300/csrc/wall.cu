@@ -7,8 +7,8 @@
 //  1. voxel key of every point (binary32 floor(p * fl(1/v)) per axis, fields
 //     offset into [0, 2^b - 2]; dropped points get the all-ones key), stable
 //     LSD radix sort of (key, index), run starts by a flag scan; each voxel's
-//     centroid is summed in binary64 in eight strands of index order, divided
-//     by the count and rounded to binary32;
+//     centroid is summed in binary64 in index order, divided by the count and
+//     rounded to binary32;
 //  2. each voxel votes for the 2-D cell of its centroid in an open-addressing
 //     hash (integer counts, so the result is order-free); a voxel is
 //     vertical when its cell holds more than min_votes voxels;
@@ -162,9 +162,32 @@ __global__ void k_wall_starts(const u64* __restrict__ keys, const uint32_t* __re
     if (i == 0 && !valid) starts[0] = 0u;  // nothing valid: nv = 0
 }
 
+// Binary32 exponents of the point's coordinates, a byte each: e_min the smallest
+// of a non-zero coordinate (255: zero), e_max the largest.
+__device__ __forceinline__ void exponents(float x, float y, float z, uint32_t& e_min, uint32_t& e_max) {
+    auto field = [](float v) { return max(__float_as_uint(v) << 1 >> 24, 1u); };
+    const uint32_t ex = field(x), ey = field(y), ez = field(z);
+    e_max = __vmaxu4(e_max, ex | ey << 8 | ez << 16);
+    e_min = __vminu4(e_min, (x != 0.0f ? ex : 255u) | (y != 0.0f ? ey : 255u) << 8 | (z != 0.0f ? ez : 255u) << 16);
+}
+// Whether sums of n < 2^31 values with these exponents are exact in binary64:
+// every value is a multiple of 2^(e_min - 150) below 2^(e_max - 126), so all
+// partial sums fit 53 bits when e_max - e_min + 24 + ceil(log2 n) <= 53.
+__device__ __forceinline__ bool sums_exact(uint32_t e_min, uint32_t e_max, uint32_t n) {
+    const int lg = n > 1 ? 32 - __clz((int)(n - 1)) : 0;
+    bool ok = true;
+#pragma unroll
+    for (int a = 0; a < 24; a += 8) ok &= (int)(e_max >> a & 255u) - (int)(e_min >> a & 255u) <= 29 - lg;
+    return ok;
+}
+
 // Eight lanes per voxel: near the sensor a voxel holds hundreds of points, and
 // one lane adding them up by dependent gathers set the kernel's time (45 us on
-// a 131k scan, 25 with eight).  Binary64 sums in eight strands, added pairwise.
+// a 131k scan, 25 with eight).  The sums are those of one lane adding in index
+// order, bit for bit: the eight strands are used where every partial sum is
+// exact (then the order does not matter; all voxels of the scan but those
+// with a coordinate within about 1e-6 m of zero), and one lane adds the others
+// up in order.
 __global__ void k_wall_centroid(const float* __restrict__ pts, const uint32_t* __restrict__ vals,
                                 const uint32_t* __restrict__ starts, const uint32_t* __restrict__ nvp,
                                 float4* __restrict__ cent) {
@@ -173,24 +196,37 @@ __global__ void k_wall_centroid(const float* __restrict__ pts, const uint32_t* _
     for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; base < nv; base += warps * 4) {
         const uint32_t v = base + (lane >> 3);
         double sx = 0.0, sy = 0.0, sz = 0.0;
-        uint32_t a = 0, b = 0;
+        uint32_t a = 0, b = 0, e_min = 0xffffffu, e_max = 0u;
         if (v < nv) {
             a = starts[v];
             b = starts[v + 1];
         }
         for (uint32_t s = a + (lane & 7); s < b; s += 8) {
             const uint32_t i = vals[s];
-            sx += (double)pts[3 * (size_t)i];
-            sy += (double)pts[3 * (size_t)i + 1];
-            sz += (double)pts[3 * (size_t)i + 2];
+            const float x = pts[3 * (size_t)i], y = pts[3 * (size_t)i + 1], z = pts[3 * (size_t)i + 2];
+            sx += (double)x;
+            sy += (double)y;
+            sz += (double)z;
+            exponents(x, y, z, e_min, e_max);
         }
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) {
             sx += __shfl_xor_sync(0xffffffffu, sx, o);
             sy += __shfl_xor_sync(0xffffffffu, sy, o);
             sz += __shfl_xor_sync(0xffffffffu, sz, o);
+            e_min = __vminu4(e_min, __shfl_xor_sync(0xffffffffu, e_min, o));
+            e_max = __vmaxu4(e_max, __shfl_xor_sync(0xffffffffu, e_max, o));
         }
         if (v < nv && (lane & 7) == 0) {
+            if (!sums_exact(e_min, e_max, b - a)) {
+                sx = sy = sz = 0.0;
+                for (uint32_t s = a; s < b; ++s) {
+                    const uint32_t i = vals[s];
+                    sx += (double)pts[3 * (size_t)i];
+                    sy += (double)pts[3 * (size_t)i + 1];
+                    sz += (double)pts[3 * (size_t)i + 2];
+                }
+            }
             const double c = (double)(b - a);
             cent[v] = make_float4((float)(sx / c), (float)(sy / c), (float)(sz / c), 0.0f);
         }
