@@ -55,12 +55,13 @@ __device__ __forceinline__ float box_eta(const Grid& g, float px, float py, floa
 // in pts (or -1) and its d2.  A box of half-width r is searched for points
 // with d2 <= T = min(tau, max_d2); every point outside the box has d2 >
 // tau, so a hit is the global nearest, and no hit with tau >= max_d2 means
-// nothing lies within max_d2.  Otherwise r doubles.  A box beyond
-// max_box_cells ends in a linear scan of the whole map (exhaustive) or in
-// `limited` with no pair.
-__device__ int nearest_within(const Grid& g, float px, float py, float pz, float max_d2, float r,
+// nothing lies within max_d2.  Otherwise r doubles.  When a box has more than
+// max_box_cells cells, the doubling starts once more, from r1 < r (so the wider
+// start, chosen for speed, costs no reach); after that such a box ends in a
+// linear scan of the whole map (exhaustive) or in `limited` with no pair.
+__device__ int nearest_within(const Grid& g, float px, float py, float pz, float max_d2, float r, float r1,
                               float& bd2, bool& limited) {
-    for (int attempt = 0; attempt < 48; ++attempt) {
+    for (int attempt = 0; attempt < 96; ++attempt) {
         const int ulx = cell_of(__fsub_rn(px, r), g.ox, g.inv_h);
         const int uhx = cell_of(__fadd_rn(px, r), g.ox, g.inv_h);
         const int uly = cell_of(__fsub_rn(py, r), g.oy, g.inv_h);
@@ -72,7 +73,12 @@ __device__ int nearest_within(const Grid& g, float px, float py, float pz, float
         const int ly = max(uly, g.wly), hy = min(uhy, g.why);
         const int lz = max(ulz, g.wlz), hz = min(uhz, g.whz);
         const int64_t ncl = (int64_t)max(hx - lx + 1, 0) * max(hy - ly + 1, 0) * max(hz - lz + 1, 0);
-        if (ncl > (int64_t)g.max_box_cells) break;
+        if (ncl > (int64_t)g.max_box_cells) {
+            if (!(r1 > 0.0f)) break;
+            r = r1;
+            r1 = 0.0f;
+            continue;
+        }
         if (tau >= 0.0f) {
             const float T = fminf(tau, max_d2);
             u64 best = EMPTY_KEY;
@@ -197,8 +203,8 @@ __device__ __forceinline__ bool pair_terms(const float* R, float px, float py, f
 }
 
 __global__ void __launch_bounds__(GICP_THREADS) k_gicp_linearize(
-    Grid g, Grid dg, int has_delta, float r0d, const float* __restrict__ map_cov, const float* __restrict__ src,
-    int64_t n, const float* __restrict__ src_cov, const float* __restrict__ pose, float max_d2, float r0,
+    Grid g, Grid dg, int has_delta, float2 r0d, const float* __restrict__ map_cov, const float* __restrict__ src,
+    int64_t n, const float* __restrict__ src_cov, const float* __restrict__ pose, float max_d2, float2 r0,
     double* __restrict__ out, int32_t* __restrict__ corr, unsigned char* __restrict__ work) {
     __shared__ double red[GICP_THREADS / 32][GICP_STRIDE];
     __shared__ unsigned ticket;
@@ -224,7 +230,7 @@ __global__ void __launch_bounds__(GICP_THREADS) k_gicp_linearize(
             if (isfinite(px) && isfinite(py) && isfinite(pz)) {
                 float bd2 = INFINITY;
                 bool limited = false;
-                const int pos = nearest_within(g, px, py, pz, max_d2, r0, bd2, limited);
+                const int pos = nearest_within(g, px, py, pz, max_d2, r0.x, r0.y, bd2, limited);
                 float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 if (pos >= 0) {
                     q = __ldg(&g.pts[pos]);
@@ -232,7 +238,7 @@ __global__ void __launch_bounds__(GICP_THREADS) k_gicp_linearize(
                 }
                 if (has_delta) {  // appended points: the nearer of the two (main index on ties)
                     float bd2d = INFINITY;
-                    const int posd = nearest_within(dg, px, py, pz, max_d2, r0d, bd2d, limited);
+                    const int posd = nearest_within(dg, px, py, pz, max_d2, r0d.x, r0d.y, bd2d, limited);
                     if (posd >= 0 && (pos < 0 || __float_as_uint(bd2d) < __float_as_uint(bd2))) {
                         q = __ldg(&dg.pts[posd]);
                         pair = (int32_t)(g.m + (int64_t)__float_as_uint(q.w));
@@ -405,7 +411,7 @@ size_t pc_gicp_work_size() {
 cudaError_t pc_launch_gicp_linearize(const pc_target_s* t, const float* map_cov, const float* src,
                                      int64_t n, const float* src_cov, const float* pose,
                                      float max_dist, double* out, int32_t* corr, void* work,
-                                     float r0, float r0d, cudaStream_t s) {
+                                     float2 r0, float2 r0d, cudaStream_t s) {
     if (n == 0) return cudaMemsetAsync(out, 0, GICP_VALS * sizeof(double), s);
     const int maxb = gicp_max_blocks();
     if (maxb < 1) return cudaErrorInvalidDevice;

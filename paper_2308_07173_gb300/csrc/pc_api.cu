@@ -836,12 +836,15 @@ pc_status pc_gicp_linearize(pc_target map, const float* map_cov_dev, const float
     // Start radius: the calibrated distance to a map point's 8th neighbour
     // (itself included).  A shorter one makes most warps search twice, a longer
     // one visits more points: 100k points against 2M, ten iterations, with the
-    // 2nd, 4th, 8th, 16th: 697, 640, 615, 755 us.
-    auto start = [](const pc_target_s* t) {
-        const float r = pc_rho0(t, (int)std::min<int64_t>(t->g.m, 8));
+    // 2nd, 4th, 8th, 16th: 697, 640, 615, 755 us.  Where that runs into
+    // max_box_cells, the search starts again from the 2nd neighbour's distance
+    // (.y), which reaches closer to the limit.
+    auto radius = [](const pc_target_s* t, int k) {
+        const float r = pc_rho0(t, (int)std::min<int64_t>(t->g.m, k));
         return r > 0.0f ? r : t->g.h;
     };
-    const float r0 = start(map), r0d = map->delta ? start(map->delta) : r0;
+    auto start = [&](const pc_target_s* t) { return make_float2(radius(t, 8), radius(t, 2)); };
+    const float2 r0 = start(map), r0d = map->delta ? start(map->delta) : r0;
     return pc_from_cuda(pc_launch_gicp_linearize(map, map_cov_dev, src_dev, n, src_cov_dev, pose_dev,
                                                  max_dist, out_dev, corr_dev, work_dev, r0, r0d,
                                                  (cudaStream_t)s));

@@ -168,7 +168,7 @@ size_t pc_gicp_work_size();
 cudaError_t pc_launch_gicp_linearize(const pc_target_s* t, const float* map_cov, const float* src,
                                      int64_t n, const float* src_cov, const float* pose,
                                      float max_dist, double* out, int32_t* corr, void* work,
-                                     float r0, float r0d, cudaStream_t s);
+                                     float2 r0, float2 r0d, cudaStream_t s);
 cudaError_t pc_launch_gicp_update(const double* lin, float lambda, float* pose, double* xi,
                                   cudaStream_t s);
 
