@@ -75,7 +75,11 @@ int pc_search_tile(const pc_target_s* t, int k, int64_t n) {
     // (each starts from the last one's radius): tiles shrink until a call has
     // as many warps as the chip holds at its 64 registers.  20k queries, k = 48
     // on a 300k map, tiles of 32 (4 warps an SM): 188 us, of 4: 96 us.
+    // Not where the exact scan may not follow (exhaustive = 0): there the radius
+    // a query starts from decides whether it is answered, and must not depend
+    // on the size of the call.
     const int most = t->tune.tile <= 0 ? 32 : std::min(t->tune.tile, 32);
+    if (!t->g.exhaustive) return most;
     return (int)std::max<int64_t>(1, std::min<int64_t>(most, n / WARP_PATH_WARPS));
 }
 

@@ -304,6 +304,19 @@ __device__ __forceinline__ bool box_allowed(const Grid& g, const WarpBox& b) {
     return b.ncl <= (int64_t)g.max_box_cells;
 }
 
+// Whether a group (k <= 32) searches a box of so many cells in so many rows.
+__device__ __forceinline__ bool group_allowed(const Grid& g, int64_t ncl, int64_t nrows) {
+    return ncl <= 4096 && nrows <= 256 && (g.dstart || ncl <= 256);
+}
+
+// Where the exact scan may not follow (exhaustive = 0), the radii decide which
+// queries are answered, so they do not follow the counts found: the group
+// search has LIMITED_RADII of them, LIMITED_START times the calibrated radius
+// and LIMITED_STEP times the one before, and k_knn_rest tries the same ones for
+// whatever a group could not sort before it widens up to max_box_cells.
+constexpr int LIMITED_RADII = 3;
+constexpr float LIMITED_START = 1.46f, LIMITED_STEP = 1.8f;
+
 template <int SLOTS>
 __device__ __forceinline__ void scan_warp_box(const Grid& g, float qx, float qy, float qz, const WarpBox& b, float tau,
                                               SearchState<SLOTS>& S, u64* pend, int k, int lane, uint32_t ibase) {
@@ -321,23 +334,35 @@ __device__ __forceinline__ void scan_warp_box(const Grid& g, float qx, float qy,
 // g and the appended-points grid dg, whose point j is g.m + j: every
 // attempt scans both grids' boxes of the same radius, filtered by the
 // smaller of their two certified taus (a point of either grid outside its
-// box lies beyond both), and the exhaustive scan covers both grids.
+// box lies beyond both), and the exhaustive scan covers both grids.  The first
+// `fixed` attempts are those of a group search under a limit (above), from rho;
+// the widening proper then starts from rho1.
 constexpr int SEARCH_OK = 0, SEARCH_LIMIT = 1, SEARCH_SHORT = 2;
 template <int SLOTS, bool DEL>
 __device__ int knn_search(const Grid& g, const Grid& dg, float qx, float qy, float qz, int k, float& rho,
-                          SearchState<SLOTS>& S, u64* pend, int lane) {
-    for (int attempt = 0; attempt < 40; ++attempt) {
+                          SearchState<SLOTS>& S, u64* pend, int lane, int fixed = 0, float rho1 = 0.0f) {
+    for (int attempt = 0; attempt < 40 + LIMITED_RADII; ++attempt) {
         const WarpBox b = warp_box(g, qx, qy, qz, rho);
         WarpBox d = b;
         float tau = b.tau;
         bool all = b.all;
+        const bool group = attempt < fixed;
+        auto allowed = [&](const Grid& gr, const WarpBox& x) {
+            return group ? group_allowed(gr, x.ncl, (int64_t)x.ey * x.ez) : box_allowed(gr, x);
+        };
+        bool may = allowed(g, b);
         if (DEL) {
             d = warp_box(dg, qx, qy, qz, rho);
             tau = fminf(tau, d.tau);
             all = all && d.all;
-            if (!box_allowed(dg, d)) break;
+            may = may && allowed(dg, d);
         }
-        if (!box_allowed(g, b)) break;
+        if (!may) {
+            if (!group) break;
+            fixed = 0;
+            rho = rho1;
+            continue;
+        }
         if (all && g.exhaustive) tau = INFINITY;  // no point lies outside the box
         state_reset(S);
         scan_warp_box(g, qx, qy, qz, b, tau, S, pend, k, lane, 0u);
@@ -345,6 +370,10 @@ __device__ int knn_search(const Grid& g, const Grid& dg, float qx, float qy, flo
         flush(S, pend, k, lane);
         if (S.kth != EMPTY_KEY) return SEARCH_OK;
         if (all && g.exhaustive) return SEARCH_SHORT;  // every point of the window was seen
+        if (group) {
+            rho = attempt + 1 < fixed ? rho * LIMITED_STEP : rho1;
+            continue;
+        }
         int found = 0;
 #pragma unroll
         for (int s = 0; s < SLOTS; ++s) found += __popc(__ballot_sync(FULL, S.L[s] != EMPTY_KEY));
@@ -744,6 +773,7 @@ __device__ void cov_row_any(const Grid& g, const Grid& dg, const int32_t* nb, in
 // registers and ran 1.35 waves of long warps.
 constexpr int MAX_ATTEMPTS = 6;
 constexpr float START = 1.4f;  // first radius over the calibrated starting radius; 1.26 and 1.54: 8 and 12 % slower
+__device__ __forceinline__ float start_factor(const Grid& g) { return g.exhaustive ? START : LIMITED_START; }
 constexpr int BATCH = 2;       // point loads a lane has in flight; 1 and 3: 3 % slower on scans
 constexpr uint32_t UNANSWERED = 0xffffffffu, UNIT_FLAG = 0x80000000u;
 constexpr uint32_t NAN_ROW = 0x7fc00000u;  // every entry of a covariance row without a value
@@ -985,7 +1015,7 @@ __device__ __forceinline__ GroupBox group_box(const Grid& g, float qx, float qy,
     b.hz = min(hz, WIN ? g.whz : g.dimz - 1);
     const int64_t nrows = (int64_t)max(b.hy - b.ly + 1, 0) * max(b.hz - b.lz + 1, 0);
     const int64_t ncl = nrows * max(b.hx - b.lx + 1, 0);
-    b.big = ncl > 4096 || nrows > 256 || (!g.dstart && ncl > 256);
+    b.big = !group_allowed(g, ncl, nrows);
     return b;
 }
 
@@ -1085,12 +1115,12 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
     {
         float r = rho0;
         if (a.probe_c > 0.0f) r = probe_radius<G, WIN>(g, finite, qx, qy, qz, k, a.probe_c, sub);
-        r *= START;
+        r *= start_factor(g);
         r2 = fminf(r * r, 1e30f);
     }
     float lo2 = 0.0f, hi2 = -1.0f;  // squared radii known to hold too few / too many (hi2 > 0)
     bool todo = finite, ok = false;
-    int w = 0, m = 0;
+    int w = 0, m = 0, wider = 0;
     float t = -1.0f;
     for (int attempt = 0; attempt < MAX_ATTEMPTS; ++attempt) {
         if (!__any_sync(FULL, todo)) break;
@@ -1133,7 +1163,11 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
         if (todo) {
             if (mm < (uint32_t)k) {  // widen; a wider box also certifies further
                 lo2 = r2;
-                const float f = fminf(fmaxf(1.7f * (float)k / (float)max(mm, 1u), 1.5f), 9.0f);
+                float f = fminf(fmaxf(1.7f * (float)k / (float)max(mm, 1u), 1.5f), 9.0f);
+                if (!g.exhaustive) {
+                    f = LIMITED_STEP * LIMITED_STEP;
+                    if (!(hi2 > 0.0f) && ++wider == LIMITED_RADII) todo = false;
+                }
                 r2 = hi2 > 0.0f ? 0.5f * (lo2 + hi2) : fminf(fmaxf(r2, 1e-6f * g.h * g.h) * f, 1e30f);
             } else if (over) {  // narrow
                 hi2 = tt;

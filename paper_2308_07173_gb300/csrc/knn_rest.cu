@@ -90,10 +90,14 @@ __device__ __forceinline__ void rest_body(const Grid& g, const Grid& dg, int64_t
                     continue;
                 }
                 const float qx = __ldg(r.q + 3 * n), qy = __ldg(r.q + 3 * n + 1), qz = __ldg(r.q + 3 * n + 2);
-                float rho = rho0 * START;
+                const float rho1 = rho0 * start_factor(g);
+                float rho = rho1;
+                if (!g.exhaustive && a.probe_c > 0.0f)
+                    rho = LIMITED_START * probe_radius<32, true>(g, true, qx, qy, qz, k, a.probe_c, lane);
                 SearchState<1> S;
                 state_reset(S);
-                const int sr = knn_search<1, DEL>(g, dg, qx, qy, qz, k, rho, S, s_pend[warp], lane);
+                const int sr = knn_search<1, DEL>(g, dg, qx, qy, qz, k, rho, S, s_pend[warp], lane,
+                                                  g.exhaustive ? 0 : LIMITED_RADII, rho1);
                 const bool ok = sr == SEARCH_OK;
                 if (!ok && lane == 0) atomicOr(g.status, sr == SEARCH_SHORT ? ST_SHORT : ST_SEARCH_LIMIT);
                 if (lane < k) {

@@ -81,3 +81,59 @@ def test_gicp_reach(gpu_lib, cells):
     assert must.sum() > 300
     assert (corr[must] >= 0).all()
     np.testing.assert_array_equal(corr[corr >= 0], oracle.knn_brute(src, mp, 1)[0][corr >= 0, 0])
+
+
+# ---------------------------------------------------------------- kNN
+@pytest.mark.parametrize("n", [3000, 24_600])
+@pytest.mark.parametrize("k", [1, 10, 20, 32])
+@pytest.mark.parametrize("cells", [8, 64, 512])
+def test_knn_reach(gpu_lib, cells, k, n):
+    """A query is answered when one of the three fixed radii (1.46, 2.63, 4.73 times the calibrated one) holds its k
+    neighbours in a box of at most 4096 cells and 256 rows, the smaller ones having held fewer."""
+    mp, q = clusters(cells, n)
+    t = gpu_lib.Target(dev(mp), cell_size=1.0, max_box_cells=cells, exhaustive=False)
+    info = t.info()
+    head = q[:3000]
+    ri, rd = oracle.knn_brute(head, mp, k)
+    d = np.sqrt(rd[:, -1])
+    hint = info["rho_hint"][k - 1]
+    r = 1.46 * 0.9 * (hint if hint > 0 else info["cell_size"])
+    must = np.zeros(len(head), bool)
+    for j in range(3):
+        ncl, rows = boxes(info, head.astype(np.float64), r * 1.8 ** j)
+        must |= (ncl <= 4096) & (rows <= 256) & (d < 0.999 * r * 1.8 ** j)
+    t.set_tune(probe=1)  # every query from the calibrated radius
+    idx, d2 = t.knn(dev(q), k)
+    t.sync_status()
+    idx, d2 = idx.cpu().numpy()[:3000], d2.cpu().numpy()[:3000]
+    t.close()
+    got = idx[:, 0] >= 0
+    assert must.sum() > 300
+    assert got[must].all()
+    np.testing.assert_array_equal(idx[got], ri[got])
+    np.testing.assert_array_equal(d2[got], rd[got])
+
+
+def test_far_query_stays_refused(gpu_lib):
+    mp = lattice(24, 24, 20)
+    t = gpu_lib.Target(dev(mp), cell_size=0.5, max_box_cells=8, exhaustive=False)
+    idx, d2 = t.knn(dev(np.array([[5e3, 0, 0]], F)), 8)
+    assert t.sync_status() == gpu_lib.PC_ERR_SEARCH_LIMIT
+    assert (idx == -1).all()
+    t.close()
+
+
+@pytest.mark.parametrize("k", [40, 64])
+def test_wide_k_does_not_depend_on_the_call(gpu_lib, k):
+    """Of 64 queries the same ones are answered alone and at the head of a call of 20,000."""
+    mp, q = clusters(k, 20_000)
+    differ = 0
+    for cells in (64, 512):
+        t = gpu_lib.Target(dev(mp), max_box_cells=cells, exhaustive=False)
+        whole = t.knn(dev(q), k)[0].cpu().numpy()
+        for at in range(0, 640, 64):
+            part = t.knn(dev(q[at:at + 64]), k)[0].cpu().numpy()
+            differ += int((part != whole[at:at + 64]).any(1).sum())
+        t.sync_status()
+        t.close()
+    assert differ == 0
