@@ -647,8 +647,8 @@ cudaError_t pc_launch_rho_hints(const float* d2, int n, int kc, float* out, cuda
 }
 
 void pc_free_grid(pc_target_s* t) {
-    void* const ps[] = {t->table, t->pts, t->xyz, t->cell_keys, t->cell_start, t->status, t->dstart, t->xcut};
-    pc_dev_free_idle(ps, 8);
+    void* const ps[] = {t->table, t->pts, t->xyz, t->cell_keys, t->cell_start, t->dstart, t->xcut};
+    pc_dev_free_idle(t->status, ps, 7);
     if (t->stage) cudaFree(t->stage);
     t->table = nullptr;
     t->pts = t->xyz = nullptr;
@@ -672,8 +672,8 @@ pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& opts, 
     Scratch sc(s);
     auto keep = [&](auto** p, size_t bytes) { return pc_dev_alloc(reinterpret_cast<void**>(p), bytes, s); };
     // persistent small buffers first
-    // status word + statistics counters (64 bytes)
-    PC_TRY(keep(&t->status, 64));
+    // status word + statistics counters (64 bytes), the target's fence
+    PC_TRY(pc_fence_alloc(reinterpret_cast<void**>(&t->status), 64));
     PC_TRY(cudaMemsetAsync(t->status, 0, 64, s));
 
     // 1. bbox + finite check

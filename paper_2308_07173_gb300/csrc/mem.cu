@@ -6,6 +6,16 @@
 // nothing uses them and gives the rest back to the device at the next
 // synchronisation; an allocation that finds no memory first gives back all of
 // it and tries again.  The pool's own calls are safe from any thread.
+//
+// A closed target's memory may still be in use on any of the caller's streams
+// (or by a graph that replays a search), so a close waits for the device, as
+// cudaFree does, through cudaFree: every target owns one small plain
+// allocation, its fence, and freeing that waits (30 ms of queued work: 30 ms).
+// cudaDeviceSynchronize instead fails, and ruins the capture, while any
+// thread captures a stream; cudaFree in relaxed mode does not.  The anchor, a
+// plain allocation that is never freed, keeps the block that fences are carved
+// from mapped: allocating and freeing a fence takes 2 + 2 us with it, 77 + 50
+// without.
 #include <mutex>
 
 #include "pc_internal.h"
@@ -13,11 +23,13 @@
 namespace {
 
 constexpr uint64_t POOL_KEEP = 256ull << 20;
+constexpr size_t ANCHOR_BYTES = 256;
 
 struct Pool {
     bool made;
     cudaMemPool_t pool;   // null: the device has no pools (plain allocations then)
     cudaStream_t frees;   // memory whose last use is known to be over is freed here
+    void* anchor;
 };
 std::mutex g_pool_mu;
 Pool g_pools[64];
@@ -34,6 +46,8 @@ Pool* current_pool() {
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
     uint64_t keep = POOL_KEEP;
+    RelaxedCapture relaxed;
+    if (cudaMalloc(&p.anchor, ANCHOR_BYTES) != cudaSuccess) cudaGetLastError();  // slower fences, nothing else
     if (cudaStreamCreateWithFlags(&p.frees, cudaStreamNonBlocking) != cudaSuccess ||
         cudaMemPoolCreate(&p.pool, &props) != cudaSuccess ||
         cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
@@ -66,13 +80,17 @@ void pc_dev_free(void* ptr, cudaStream_t s) {
     else cudaFree(ptr);
 }
 
-void pc_dev_free_idle(void* const* ptrs, int n) {
+cudaError_t pc_fence_alloc(void** out, size_t bytes) {
+    if (!current_pool()) return cudaErrorInvalidDevice;  // the anchor first
+    RelaxedCapture relaxed;
+    return cudaMalloc(out, bytes);
+}
+
+void pc_dev_free_idle(void* fence, void* const* ptrs, int n) {
     Pool* p = current_pool();
-    if (!p) return;
-    // as cudaFree does: the caller's streams may still use them.  Where that is
-    // refused (this thread is capturing), the memory stays allocated, as it did
-    // when cudaFree was refused.
-    if (p->pool && cudaDeviceSynchronize() != cudaSuccess) {
+    if (!p || !fence) return;  // without a fence nothing else was allocated
+    RelaxedCapture relaxed;
+    if (cudaFree(fence) != cudaSuccess) {  // the context is lost, and the memory with it
         cudaGetLastError();
         return;
     }

@@ -285,6 +285,7 @@ void pc_destroy_target(pc_target t) {
     if (!t || !live(t)) return;
     untrack(t);
     DeviceGuard dg(t->device);
+    RelaxedCapture relaxed;
     free_delta(t);
     pc_free_grid(t);
     t->magic = PC_MAGIC_DEAD;

@@ -111,11 +111,22 @@ inline void pc_clear_window(pcdev::Grid& g) {
 }
 
 // mem.cu: device memory of targets on the current device, ready for use in
-// the order of stream s.  pc_dev_free: after the work queued on s;
-// pc_dev_free_idle: after a device synchronisation, for any stream's users.
+// the order of stream s.  pc_dev_free: after the work queued on s.
 cudaError_t pc_dev_alloc(void** out, size_t bytes, cudaStream_t s);
 void pc_dev_free(void* ptr, cudaStream_t s);
-void pc_dev_free_idle(void* const* ptrs, int n);
+// A target's fence, usable as memory; freeing it waits for the device.
+// pc_dev_free_idle frees it and then the pool memory at ptrs, for any stream's
+// users and while any thread captures.
+cudaError_t pc_fence_alloc(void** out, size_t bytes);
+void pc_dev_free_idle(void* fence, void* const* ptrs, int n);
+
+// Calls that wait for the device, or allocate, leave captures in progress alone.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    RelaxedCapture(const RelaxedCapture&) = delete;
+};
 
 // grid_build.cu
 pc_status pc_build_grid(const float* xyz, int64_t M, const pc_build_opts& o, cudaStream_t s,

@@ -1,0 +1,84 @@
+"""Device memory of targets: closing beside captures in progress."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def cloud(n, seed=0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.rand((n, 3), device="cuda", generator=g) * torch.tensor([300.0, 200.0, 3.0], device="cuda")
+
+
+SETUP = """
+import sys, threading, torch
+from paper_2308_07173_gb300 import pc
+cloud = lambda n: torch.rand((n, 3), device="cuda") * torch.tensor([300.0, 200.0, 3.0], device="cuda")
+free = lambda: torch.cuda.mem_get_info()[0]
+big, q = cloud(20_000_000), cloud(1000)
+t = pc.Target(q)
+want, _ = t.knn(q, 5)
+idx, d2 = torch.empty_like(want), torch.empty((1000, 5), device="cuda")
+torch.cuda.synchronize()
+before = free()
+other = pc.Target(big)
+"""
+
+CLOSE = {
+    "another thread": """
+def close():
+    th = threading.Thread(target=other.close)
+    th.start()
+    th.join()
+""",
+    "this thread": """
+def close():
+    other.close()
+""",
+}
+
+CAPTURE = """
+graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+with torch.cuda.graph(graph, stream=s, capture_error_mode=sys.argv[1]):
+    close()
+    t.knn(q, 5, idx, d2, stream=s)
+graph.replay()
+torch.cuda.synchronize()
+assert torch.equal(idx, want)
+assert before - free() <= (256 + 64) << 20, (before - free()) >> 20
+"""
+
+
+def child(code, *args):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code, *args], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-1500:]
+
+
+@pytest.mark.parametrize("mode", ["thread_local", "global", "relaxed"])
+@pytest.mark.parametrize("who", list(CLOSE))
+def test_close_beside_a_capture(gpu_lib, who, mode):
+    """The capture stays valid and the memory comes back."""
+    child(SETUP + CLOSE[who] + CAPTURE, mode)
+
+
+def test_close_waits_for_searches_on_other_streams(gpu_lib):
+    t = gpu_lib.Target(cloud(200_000))
+    q = cloud(300_000, 1)
+    want = t.knn(q, 20)[0]
+    idx, d2 = torch.empty_like(want), torch.empty((len(q), 20), device="cuda")
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(40_000_000)
+    t.knn(q, 20, idx, d2, stream=s)
+    done = torch.cuda.Event()
+    done.record(s)
+    t.close()
+    assert done.query()
+    assert torch.equal(idx, want)
