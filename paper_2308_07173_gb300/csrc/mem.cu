@@ -2,10 +2,10 @@
 // per device.  A build makes about 25 allocations; through cudaMalloc and
 // cudaFree each took 40-90 us (and every cudaFree waited for the device): with them
 // a 131k-point target took 1.19 ms to build and 0.25 ms to close, with the pool
-// 0.55 and 0.01.  The pool keeps at most POOL_KEEP bytes when
-// nothing uses them and gives the rest back to the device at the next
-// synchronisation; an allocation that finds no memory first gives back all of
-// it and tries again.  The pool's own calls are safe from any thread.
+// 0.55 and 0.01.  When a build or a close returns, the pool keeps at most
+// POOL_KEEP unused bytes; every allocation of the library that finds no memory
+// first gives those back to the device and tries again.  The pool's own calls
+// are safe from any thread.
 //
 // A closed target's memory may still be in use on any of the caller's streams
 // (or by a graph that replays a search), so a close waits for the device, as
@@ -57,6 +57,14 @@ Pool* current_pool() {
     return &p;
 }
 
+// The pool's unused memory back to the device.
+void give_back(Pool* p) {
+    if (!p || !p->pool) return;
+    RelaxedCapture relaxed;
+    cudaStreamSynchronize(p->frees);
+    cudaMemPoolTrimTo(p->pool, 0);
+}
+
 }  // namespace
 
 cudaError_t pc_dev_alloc(void** out, size_t bytes, cudaStream_t s) {
@@ -67,7 +75,7 @@ cudaError_t pc_dev_alloc(void** out, size_t bytes, cudaStream_t s) {
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         cudaStreamSynchronize(s);
-        cudaMemPoolTrimTo(p->pool, 0);
+        give_back(p);
         e = cudaMallocFromPoolAsync(out, bytes, p->pool, s);
     }
     return e;
@@ -80,10 +88,20 @@ void pc_dev_free(void* ptr, cudaStream_t s) {
     else cudaFree(ptr);
 }
 
+cudaError_t pc_plain_alloc(void** out, size_t bytes) {
+    cudaError_t e = cudaMalloc(out, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        give_back(current_pool());
+        e = cudaMalloc(out, bytes);
+    }
+    return e;
+}
+
 cudaError_t pc_fence_alloc(void** out, size_t bytes) {
     if (!current_pool()) return cudaErrorInvalidDevice;  // the anchor first
     RelaxedCapture relaxed;
-    return cudaMalloc(out, bytes);
+    return pc_plain_alloc(out, bytes);
 }
 
 void pc_dev_free_idle(void* fence, void* const* ptrs, int n) {
@@ -99,4 +117,6 @@ void pc_dev_free_idle(void* fence, void* const* ptrs, int n) {
         if (p->pool) cudaFreeAsync(ptrs[i], p->frees);
         else cudaFree(ptrs[i]);
     }
+    // the pool gives back what is above POOL_KEEP at a synchronisation
+    if (p->pool) cudaStreamSynchronize(p->frees);
 }

@@ -111,8 +111,8 @@ pc_status calibrate_rho(pc_target_s* t, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, hints, sizeof(h), cudaMemcpyDeviceToHost, s);
     // the status word and statistics start clean (a capped search here only skips that sample)
     if (e == cudaSuccess) e = cudaMemsetAsync(t->status, 0, 64, s);
-    const cudaError_t e2 = cudaStreamSynchronize(s);
     pc_dev_free(buf, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);  // the pool gives back what it need not keep
     if (e != cudaSuccess || e2 != cudaSuccess) return pc_from_cuda(e != cudaSuccess ? e : e2);
     std::memcpy(t->rho_hint, h, 64 * sizeof(float));
     // spread of the distances at k = min(kc, 16): a map whose density varies
@@ -129,7 +129,7 @@ pc_status ensure_stage(pc_target_s* t, size_t bytes) {
         t->stage_bytes = 0;
     }
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
+    cudaError_t e = pc_plain_alloc(&p, bytes);
     if (e != cudaSuccess) return pc_from_cuda(e);
     t->stage = p;
     t->stage_bytes = bytes;
@@ -167,6 +167,7 @@ static pc_status build_target_internal(const float* xyz, int64_t M, const pc_bui
         if (like) {
             std::memcpy(t->rho_hint, like->rho_hint, sizeof(t->rho_hint));
             t->uneven = like->uneven;
+            r = pc_from_cuda(cudaStreamSynchronize(st));  // the pool gives back what it need not keep
         }
         else r = calibrate_rho(t, st);
     }
@@ -479,7 +480,7 @@ pc_status pc_batch_plan(pc_target t, const pc_scan* scans, int n_scans, int k, f
     b->warps = sh.warps;
     b->total_tiles = sh.tiles;
     b->total_queries = sh.queries;
-    cudaError_t e = cudaMalloc(&b->scans_dev, sizeof(ScanDesc) * n_scans);
+    cudaError_t e = pc_plain_alloc(reinterpret_cast<void**>(&b->scans_dev), sizeof(ScanDesc) * n_scans);
     if (e == cudaSuccess)
         e = cudaMemcpy(b->scans_dev, hs.data(), sizeof(ScanDesc) * n_scans, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -692,7 +693,7 @@ pc_status pc_target_append(pc_target t, const float* xyz_dev, int64_t n, pc_stre
     if (tot > t->delta_cap) {  // grow the appended-points array (doubling)
         const int64_t cap = std::max<int64_t>(tot, 2 * t->delta_cap);
         float* p = nullptr;
-        cudaError_t e = cudaMalloc(&p, sizeof(float) * 3 * cap);
+        cudaError_t e = pc_plain_alloc(reinterpret_cast<void**>(&p), sizeof(float) * 3 * cap);
         if (e != cudaSuccess) return pc_from_cuda(e);
         if (t->delta_m > 0)
             e = cudaMemcpyAsync(p, t->delta_xyz, sizeof(float) * 3 * t->delta_m, cudaMemcpyDeviceToDevice, st);
@@ -733,7 +734,7 @@ pc_status pc_target_compact(pc_target t, pc_stream s) {
     cudaStream_t st = (cudaStream_t)s;
     const int64_t tot = t->g.m + t->delta_m;
     float* all = nullptr;
-    cudaError_t e = cudaMalloc(&all, sizeof(float) * 3 * tot);
+    cudaError_t e = pc_plain_alloc(reinterpret_cast<void**>(&all), sizeof(float) * 3 * tot);
     if (e != cudaSuccess) return pc_from_cuda(e);
     e = pc_launch_pack_xyz(t, all, st);
     pc_target_s* n = nullptr;

@@ -114,6 +114,8 @@ inline void pc_clear_window(pcdev::Grid& g) {
 // the order of stream s.  pc_dev_free: after the work queued on s.
 cudaError_t pc_dev_alloc(void** out, size_t bytes, cudaStream_t s);
 void pc_dev_free(void* ptr, cudaStream_t s);
+// cudaMalloc that asks the pool for its unused memory before it fails.
+cudaError_t pc_plain_alloc(void** out, size_t bytes);
 // A target's fence, usable as memory; freeing it waits for the device.
 // pc_dev_free_idle frees it and then the pool memory at ptrs, for any stream's
 // users and while any thread captures.

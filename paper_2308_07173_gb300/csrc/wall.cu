@@ -666,7 +666,7 @@ pc_status pc_wall_create(int64_t max_points, const pc_wall_opts* opts, pc_wall* 
     const size_t o_cminx = take(4 * N), o_cmaxx = take(4 * N), o_cminy = take(4 * N), o_cmaxy = take(4 * N),
                  o_ccount = take(4 * N), o_nvert = take(4), o_out = take(sizeof(WallOut)), o_pick = take(8),
                  o_partial = take(sizeof(double) * FIT_BLOCKS * FIT_VALS), o_ticket = take(4);
-    cudaError_t e = cudaMalloc(&w->mem, off);
+    cudaError_t e = pc_plain_alloc(&w->mem, off);
     if (e != cudaSuccess) {
         delete w;
         return pc_from_cuda(e);

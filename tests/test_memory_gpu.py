@@ -1,4 +1,5 @@
-"""Device memory of targets: closing beside captures in progress."""
+"""Device memory of targets: what builds and closed handles give back, and closing
+beside captures in progress."""
 import os
 import subprocess
 import sys
@@ -9,10 +10,41 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
+MB = 1 << 20
+KEPT = 256 * MB + 32 * MB  # the pool's unused bytes, and the granularity of allocations
+
+
+def free():
+    return torch.cuda.mem_get_info()[0]
+
 
 def cloud(n, seed=0):
     g = torch.Generator(device="cuda").manual_seed(seed)
     return torch.rand((n, 3), device="cuda", generator=g) * torch.tensor([300.0, 200.0, 3.0], device="cuda")
+
+
+def test_builds_and_closed_targets_keep_little(gpu_lib):
+    p = cloud(20_000_000)
+    gpu_lib.Target(p[:1000]).close()
+    torch.cuda.synchronize()
+    before = free()
+    t = gpu_lib.Target(p)
+    assert before - free() <= t.info()["device_bytes"] + KEPT
+    t.append(p[:5_000_000])
+    assert before - free() <= t.info()["device_bytes"] + KEPT
+    t.close()
+    assert before - free() <= KEPT
+
+
+def test_other_allocations_take_what_the_pool_keeps(gpu_lib):
+    gpu_lib.Target(cloud(20_000_000)).close()
+    torch.cuda.empty_cache()
+    hold = torch.empty(free() - 80 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        gpu_lib.WallDetector(1_000_000).close()  # 135 MB
+    finally:
+        del hold
+        torch.cuda.empty_cache()
 
 
 SETUP = """
