@@ -136,6 +136,16 @@ pc_status ensure_stage(pc_target_s* t, size_t bytes) {
     return PC_OK;
 }
 
+// Whether s captures.  Builds, appends and compactions cannot be captured and
+// refuse before anything is queued or allocated: a copy left in the caller's
+// graph would write the target's memory at every replay.
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -147,12 +157,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 // searched with one trial radius, and an append costs one grid build.
 static pc_status build_target_internal(const float* xyz, int64_t M, const pc_build_opts& o, cudaStream_t st,
                                        pc_target_s** out, const pc_target_s* like = nullptr) {
-    // a build cannot be captured: refuse before anything is queued or allocated
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return PC_ERR_CUDA;
-    }
+    if (capturing(st)) return PC_ERR_CUDA;
     pc_target_s* t = new (std::nothrow) pc_target_s();
     if (!t) return PC_ERR_OOM;
     std::memset(t, 0, sizeof(*t));
@@ -690,6 +695,7 @@ pc_status pc_target_append(pc_target t, const float* xyz_dev, int64_t n, pc_stre
     if (t->g.m + tot >= ((int64_t)1 << 31)) return PC_ERR_INVALID_ARG;
     DeviceGuard dg(t->device);
     cudaStream_t st = (cudaStream_t)s;
+    if (capturing(st)) return PC_ERR_CUDA;
     if (tot > t->delta_cap) {  // grow the appended-points array (doubling)
         const int64_t cap = std::max<int64_t>(tot, 2 * t->delta_cap);
         float* p = nullptr;
@@ -732,6 +738,7 @@ pc_status pc_target_compact(pc_target t, pc_stream s) {
     if (!t->delta) return PC_OK;
     DeviceGuard dg(t->device);
     cudaStream_t st = (cudaStream_t)s;
+    if (capturing(st)) return PC_ERR_CUDA;
     const int64_t tot = t->g.m + t->delta_m;
     float* all = nullptr;
     cudaError_t e = pc_plain_alloc(reinterpret_cast<void**>(&all), sizeof(float) * 3 * tot);

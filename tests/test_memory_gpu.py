@@ -114,3 +114,28 @@ def test_close_waits_for_searches_on_other_streams(gpu_lib):
     t.close()
     assert done.query()
     assert torch.equal(idx, want)
+
+
+@pytest.mark.parametrize("mode", ["thread_local", "global", "relaxed"])
+def test_append_and_compact_refuse_a_capture_and_leave_nothing_in_it(gpu_lib, mode):
+    p = cloud(1014, 2)
+    t = gpu_lib.Target(p[:1000])
+    t.append(p[1000:1010])
+    t.append(p[1010:1011])  # room for 20: the next ones do not allocate
+    graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    x = torch.zeros(4, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=s, capture_error_mode=mode):
+        x.add_(1)
+        for refused in (lambda: t.append(p[1013:1014], stream=s), lambda: t.compact(stream=s)):
+            with pytest.raises(gpu_lib.PcError) as e:
+                refused()
+            assert e.value.code == gpu_lib.PC_ERR_CUDA
+    t.append(p[1011:1012])
+    graph.replay()
+    torch.cuda.synchronize()
+    t.append(p[1012:1013])  # the grid of appended points is built again
+    idx, d2 = t.knn(p[1011:1013].contiguous(), 1)
+    assert idx.flatten().tolist() == [1011, 1012] and (d2 == 0).all()
+    assert (x == 1).all()
+    t.close()
