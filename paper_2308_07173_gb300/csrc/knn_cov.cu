@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 
 #include "knn_kernels.cuh"
 
@@ -44,6 +45,13 @@ int clamp_warps(int w) { return w <= 0 ? 4 : (w > 8 ? 8 : w); }
 // 42 / 33, 51 / 55; uniform box, k = 20 46 / 34, 53 / 50, 78 / 80.
 int group_lanes(int64_t n) { return n <= 24576 ? 8 : 4; }
 
+void* search_kernel(int form, bool windowed, int mode, int cov, int group) {
+    return windowed    ? pc_knn_kernel_win(form, mode, cov, group)
+           : form == 2 ? pc_knn_kernel_union(mode, cov, group)
+           : form == 1 ? pc_knn_kernel_batch(mode, cov, group)
+                       : knn_kernel<0, false>(mode, cov, group);
+}
+
 // Launches the search kernel of (form, mode, covariance kind, window) over
 // its work items: one per one-warp block of the group search, one per warp of
 // the warp path.
@@ -51,10 +59,7 @@ cudaError_t launch_form(int form, const Grid& g, int mode, int cov, int64_t tile
                         cudaStream_t s) {
     if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
     const int group = mode < 2 ? 32 / tile : 1;
-    void* kern = g.windowed ? pc_knn_kernel_win(form, mode, cov, group)
-               : form == 2  ? pc_knn_kernel_union(mode, cov, group)
-               : form == 1  ? pc_knn_kernel_batch(mode, cov, group)
-                            : knn_kernel<0, false>(mode, cov, group);
+    void* kern = search_kernel(form, g.windowed != 0, mode, cov, group);
     if (mode < 2) warps = 1;
     return cudaLaunchKernel(kern, dim3((unsigned)((tiles + warps - 1) / warps)), dim3(32 * warps), args, 0, s);
 }
@@ -66,6 +71,31 @@ TileArgs tile_args(const pc_target_s* t, const CovKernel& ck, int k, float eps, 
 }
 
 }  // namespace
+
+// A kernel that has not run yet is loaded by its first launch, which takes
+// device memory (2 MB at a time) and 0.7 ms more: too late for the entries that
+// promise not to allocate, and for the first scan served.
+cudaError_t pc_knn_prepare() {
+    static std::mutex mu;
+    static uint64_t done = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || dev < 0 || dev >= 64) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    if (done >> dev & 1) return cudaSuccess;
+    cudaFuncAttributes at;
+    for (int form = 0; form < 3; ++form)
+        for (int win = 0; win < 2; ++win)
+            for (int mode = 0; mode < 3; ++mode)
+                for (int cov = 0; cov < (mode == 2 ? 2 : 3); ++cov)
+                    for (int group = 4; group <= (mode == 2 ? 4 : 8); group += 4)
+                        if ((e = cudaFuncGetAttributes(&at, search_kernel(form, win != 0, mode, cov, group))) !=
+                            cudaSuccess)
+                            return e;
+    if ((e = pc_rest_prepare()) != cudaSuccess) return e;
+    done |= 1ull << dev;
+    return cudaSuccess;
+}
 
 constexpr int64_t WARP_PATH_WARPS = 152 * 32;
 

@@ -153,6 +153,13 @@ cudaError_t launch(void (*kern)(P...), int64_t tiles, cudaStream_t s, P... args)
 
 }  // namespace
 
+cudaError_t pc_rest_prepare() {
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, k_knn_rest<false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, k_knn_rest<true>);
+    return e == cudaSuccess ? cudaFuncGetAttributes(&at, k_knn_rest_batch) : e;
+}
+
 cudaError_t pc_launch_rest(const Grid& g, const Grid* dg, const float* q, int64_t N, int tile, const TileArgs& a,
                            float rho0, int32_t* idx, float* d2, float* cov, cudaStream_t s) {
     return launch<Grid, Grid, const float*, int64_t, int, TileArgs, float, int32_t*, float*, float*>(

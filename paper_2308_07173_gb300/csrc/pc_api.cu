@@ -158,6 +158,8 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 static pc_status build_target_internal(const float* xyz, int64_t M, const pc_build_opts& o, cudaStream_t st,
                                        pc_target_s** out, const pc_target_s* like = nullptr) {
     if (capturing(st)) return PC_ERR_CUDA;
+    const cudaError_t prepared = pc_knn_prepare();
+    if (prepared != cudaSuccess) return pc_from_cuda(prepared);
     pc_target_s* t = new (std::nothrow) pc_target_s();
     if (!t) return PC_ERR_OOM;
     std::memset(t, 0, sizeof(*t));

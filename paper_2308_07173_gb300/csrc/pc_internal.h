@@ -159,6 +159,10 @@ void* pc_knn_kernel_union_win(int mode, int cov, int group);
 // knn_cov.cu.  Outputs may be device or mapped page-locked host memory.
 cudaError_t pc_launch_knn(const pc_target_s* t, const float* q, int64_t N, int k, float eps,
                           int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s, bool host_cov = false);
+// Loads every search kernel on the current device (once; called by the first
+// build, so that no search or capture is the first to launch one).
+cudaError_t pc_knn_prepare();
+cudaError_t pc_rest_prepare();
 // Queries of one work item of a search over n queries (k <= 32: a unit of the
 // group search; else the tune's tile).
 int pc_search_tile(const pc_target_s* t, int k, int64_t n);

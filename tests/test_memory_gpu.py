@@ -1,5 +1,5 @@
-"""Device memory of targets: what builds and closed handles give back, and closing
-beside captures in progress."""
+"""Device memory of targets: what builds and closed handles give back, closing
+beside captures in progress, and entries that take no memory."""
 import os
 import subprocess
 import sys
@@ -114,6 +114,23 @@ def test_close_waits_for_searches_on_other_streams(gpu_lib):
     t.close()
     assert done.query()
     assert torch.equal(idx, want)
+
+
+def test_first_noalloc_call_takes_no_memory(gpu_lib):
+    child("""
+import torch
+from paper_2308_07173_gb300 import pc
+p, q = torch.rand((200_000, 3), device="cuda") * 50, torch.rand((50_000, 3), device="cuda") * 50
+t = pc.Target(p)
+o = (torch.empty((50_000, 20), dtype=torch.int32, device="cuda"), torch.empty((50_000, 20), device="cuda"),
+     torch.empty((50_000, 6), device="cuda"))
+torch.cuda.synchronize()
+before = torch.cuda.mem_get_info()[0]
+scan = pc.pc_scan(q.data_ptr(), 50_000, *(x.data_ptr() for x in o))
+assert pc.pc_batch_run_noalloc(t.handle, [scan], 20, 1e-3, 0) == pc.PC_OK
+torch.cuda.synchronize()
+assert torch.cuda.mem_get_info()[0] == before
+""")
 
 
 @pytest.mark.parametrize("mode", ["thread_local", "global", "relaxed"])
