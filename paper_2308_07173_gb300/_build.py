@@ -21,7 +21,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpc.so")
 
 SOURCES = ["knn_cov.cu", "knn_window.cu", "knn_batch.cu", "knn_batch_win.cu", "knn_union.cu", "knn_union_win.cu",
-           "knn_rest.cu", "pc_api.cu", "grid_build.cu", "mem.cu", "noalloc.cu", "gicp.cu", "wall.cu", "delta.cu"]
+           "knn_host.cu", "knn_host_win.cu", "knn_rest.cu", "pc_api.cu", "grid_build.cu", "mem.cu", "noalloc.cu", "gicp.cu", "wall.cu", "delta.cu"]
 HEADERS = ["pc_device.cuh", "pc_internal.h", "pc_search.cuh", "knn_kernels.cuh"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

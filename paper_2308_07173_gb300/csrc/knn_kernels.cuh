@@ -757,7 +757,8 @@ __device__ void cov_row_any(const Grid& g, const Grid& dg, const int32_t* nb, in
 //    within 2^(TB-1) ulps; a group that finds two neighbours in one such
 //    bucket is put in exact (d2, index) order by an insertion sort.
 // 4. Rows are written by the warp as one contiguous block; three lanes of
-//    the group carry the covariance sums.
+//    the group carry the covariance sums.  (Into host memory, by a block of
+//    four warps: k_knn_host.)
 //
 // k_knn_rest follows every launch.  It turns the covariances into normals and
 // C' (eps >= 0), one query per lane, and answers the queries that no attempt
@@ -1077,12 +1078,13 @@ __device__ __forceinline__ float group_moments(float* c, const TileArgs& a, floa
 // One unit of cnt <= 32 / G queries on one warp.  With DEL the search covers
 // the union of the main grid g and the grid dg of appended points (point j of
 // dg is g.m + j): both grids' boxes are walked, filtered by the smaller of
-// their certified taus, and list entries from dg carry DTAG.  Outputs may be
-// device memory or mapped host memory: rows and covariances are written as
-// contiguous blocks either way.
-template <int CAP, int G, int COV, bool WIN, bool DEL>
-__device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const float* __restrict__ q, int64_t n0,
-                                           int cnt, const TileArgs& a, float rho0, int32_t* __restrict__ idx,
+// their certified taus, and list entries from dg carry DTAG.  idx, d2 and cov
+// point at the unit's own rows.  HOST: they are in shared memory, the
+// covariances are finished here and the caller sets the mark; returns whether
+// the unit has queries left for k_knn_rest.
+template <int CAP, int G, int COV, bool WIN, bool DEL, bool HOST = false>
+__device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const float* __restrict__ q, int cnt,
+                                           const TileArgs& a, float rho0, int32_t* __restrict__ idx,
                                            float* __restrict__ d2, float* __restrict__ cov, unsigned char* smem) {
     constexpr int SLOTS = lane_slots(CAP, G), WQ = 32 / G, NN = CAP / G;
     constexpr int TB = SLOTS * G <= 64 ? 6 : 7;
@@ -1093,7 +1095,7 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
     // k_knn_rest may be set up while the last blocks run (it waits for them)
     cudaTriggerProgrammaticLaunchCompletion();
     const int k = a.k;
-    const int lane = threadIdx.x, sub = lane & (G - 1);
+    const int lane = HOST ? threadIdx.x & 31 : threadIdx.x, sub = lane & (G - 1);
     float* const ld = reinterpret_cast<float*>(smem);
     uint32_t* const lp = reinterpret_cast<uint32_t*>(smem + SLOTS * 32 * 4);
     uint32_t* const kb = reinterpret_cast<uint32_t*>(smem + SLOTS * 32 * 8);
@@ -1102,7 +1104,7 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
     const bool active = qi < cnt;
     float qx = 0.0f, qy = 0.0f, qz = 0.0f;
     if (active) {
-        const float* p = q + 3 * (n0 + qi);
+        const float* p = q + 3 * qi;
         qx = __ldg(p);
         qy = __ldg(p + 1);
         qz = __ldg(p + 2);
@@ -1298,8 +1300,7 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
     const unsigned badm = finm & ~okm;
     const bool with_cov = COV && cov != nullptr;
     {
-        uint32_t* const d2b = reinterpret_cast<uint32_t*>(d2) + n0 * k;
-        int32_t* const ib = idx + n0 * k;
+        uint32_t* const d2b = reinterpret_cast<uint32_t*>(d2);
         const uint32_t inv = (65536u + (uint32_t)k - 1u) / (uint32_t)k;  // e / k for e < 8 * 32
         float nx[ROUNDS], ny[ROUNDS], nz[ROUNDS];
         int to[ROUNDS];
@@ -1325,8 +1326,8 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
                 } else if (finm >> (qe * G) & 1u) {
                     dv = UNANSWERED;
                 }
-                if (e == 0 && badm) dv |= UNIT_FLAG;
-                ib[e] = iv;
+                if (!HOST && e == 0 && badm) dv |= UNIT_FLAG;
+                idx[e] = iv;
                 d2b[e] = dv;
             }
         }
@@ -1352,7 +1353,7 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
     if (with_cov) {
         float uu, uv;
         const float total = group_moments<CS, KMAX, G, COV == 2>(ld + qi, a, qx, qy, qz, sub, uu, uv);
-        float* const sc = reinterpret_cast<float*>(kb);  // the keys are done with
+        float* const sc = HOST ? cov : reinterpret_cast<float*>(kb);  // the keys are done with
         const bool some = ok && total > 0.0f && isfinite(total);
         const float nan = __uint_as_float(NAN_ROW);
         if (sub < 3) {  // xx, xy; yy, yz; zz, xz
@@ -1360,12 +1361,13 @@ __device__ __forceinline__ void group_unit(const Grid& g, const Grid& dg, const 
             sc[6 * qi + (sub == 0 ? 1 : sub == 1 ? 4 : 2)] = some ? uv : nan;
         }
         __syncwarp();
-        if (a.finish) {
+        if constexpr (HOST) {
             if (sub == 0 && some) cov_regularise(sc + 6 * qi, a.eps);
-            __syncwarp();
+        } else {
+            for (int i = lane; i < 6 * cnt; i += 32) cov[i] = sc[i];
         }
-        for (int i = lane; i < 6 * cnt; i += 32) cov[6 * n0 + i] = sc[i];
     }
+    return badm != 0u;
 }
 
 // k > 32: the warp-cooperative search for each query of the tile in turn.
@@ -1444,7 +1446,8 @@ __device__ __forceinline__ void process_tile(const Grid& g, const Grid& dg, cons
                                              float* __restrict__ d2, float* __restrict__ cov) {
     if constexpr (CAP > 0) {
         __shared__ __align__(16) unsigned char smem[group_warp_smem(CAP, G)];
-        group_unit<CAP, G, COV, WIN, DEL>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov, smem);
+        group_unit<CAP, G, COV, WIN, DEL>(g, dg, q + 3 * n0, cnt, a, rho0, idx + n0 * a.k, d2 + n0 * a.k,
+                                          cov ? cov + 6 * n0 : nullptr, smem);
     } else {
         __shared__ u64 pend[8][64];
         warp_tile<COV != 0, DEL>(g, dg, q, n0, cnt, a, rho0, idx, d2, cov, pend[threadIdx.x >> 5], threadIdx.x & 31);
@@ -1492,6 +1495,76 @@ __global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
     process_tile<CAP, G, COV, WIN, true>(g, dg, q, n0, (int)min((int64_t)tile, N - n0), a, rho0, idx, d2, cov);
 }
 
+// Outputs in mapped host memory (k <= 32).  A block of four warps answers
+// HOST_WARPS units (32 queries, or 16 with eight lanes each), stages their rows
+// in shared memory and writes each array's rows as one block of 16-byte
+// vectors where the row base allows it.  Bounded by the host link (186 GB/s of
+// plain copies), which wants wide stores and long blocks.  A step of 1.45M
+// points, k = 20, 184 bytes each, and saturated served throughput (three steps
+// in flight):
+//   one warp, 4-byte stores in blocks of 640 bytes   2126 us  126 GB/s  6.94e8 points/s
+//   one warp, 16-byte vectors                        1822     147       8.07e8
+//   two warps, blocks of 1280 bytes                  1712     156       8.64e8
+//   four warps, blocks of 2560 bytes                 1648     162       8.92e8
+// (Eight would not fit 48 KB.)  The block has one mark: k_knn_rest reads them
+// back over the link, and one per unit cost 2 %.  Normals on 8 of 32 lanes
+// cost nothing here.
+constexpr int HOST_WARPS = 4;
+__host__ __device__ constexpr size_t host_stage_bytes(int tile, int k) {
+    return (size_t)tile * (2 * k + 6) * sizeof(uint32_t);
+}
+
+// n words from shared to global or host memory, by all threads of the block.
+__device__ __forceinline__ void copy_rows(void* __restrict__ to, const uint32_t* __restrict__ from, int n) {
+    uint32_t* const dst = static_cast<uint32_t*>(to);
+    const int wide = ((reinterpret_cast<uintptr_t>(to) | reinterpret_cast<uintptr_t>(from)) & 15) == 0 ? n >> 2 : 0;
+    for (int i = threadIdx.x; i < wide; i += blockDim.x)
+        reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(from)[i];
+    for (int i = 4 * wide + threadIdx.x; i < n; i += blockDim.x) dst[i] = from[i];
+}
+
+template <int CAP, int G, int COV, bool WIN>
+__device__ __forceinline__ void host_tile(const Grid& g, const float* __restrict__ q, int64_t n0, int cnt,
+                                          const TileArgs& a, float rho0, int32_t* __restrict__ idx,
+                                          float* __restrict__ d2, float* __restrict__ cov) {
+    constexpr int WQ = 32 / G, TILE = HOST_WARPS * WQ;
+    __shared__ __align__(16) unsigned char smem[HOST_WARPS][group_warp_smem(CAP, G)];
+    extern __shared__ __align__(16) uint32_t stage[];  // idx rows, d2 rows, covariances of the tile
+    const int w = threadIdx.x >> 5, k = a.k, first = w * WQ;
+    uint32_t* const sd = stage + TILE * k;
+    uint32_t* const sc = sd + TILE * k;
+    const bool left = group_unit<CAP, G, COV, WIN, false, true>(
+        g, g, q + 3 * (n0 + first), min(max(cnt - first, 0), WQ), a, rho0, reinterpret_cast<int32_t*>(stage) + first * k,
+        reinterpret_cast<float*>(sd) + first * k, cov ? reinterpret_cast<float*>(sc) + 6 * first : nullptr, smem[w]);
+    if (__syncthreads_or(left) && threadIdx.x == 0) sd[0] |= UNIT_FLAG;  // copied by thread 0
+    copy_rows(idx + n0 * k, stage, cnt * k);
+    copy_rows(d2 + n0 * k, sd, cnt * k);
+    if (COV && cov != nullptr) copy_rows(cov + 6 * n0, sc, cnt * 6);
+}
+
+constexpr int host_blocks(int cap) { return cap == 32 ? 8 : 5; }  // what shared memory and 64 (102) registers allow
+
+template <int CAP, int G, int COV, bool WIN>
+__global__ void __launch_bounds__(32 * HOST_WARPS, host_blocks(CAP))
+    k_knn_host(Grid g, const float* __restrict__ q, int64_t N, int tile, TileArgs a, float rho0,
+               int32_t* __restrict__ idx, float* __restrict__ d2, float* __restrict__ cov) {
+    const int64_t t = work_item<CAP>((N + tile - 1) / tile, a.last_first);
+    if (t < 0) return;
+    const int64_t n0 = t * tile;
+    host_tile<CAP, G, COV, WIN>(g, q, n0, (int)min((int64_t)tile, N - n0), a, rho0, idx, d2, cov);
+}
+
+template <int CAP, int G, int COV, bool WIN>
+__global__ void __launch_bounds__(32 * HOST_WARPS, host_blocks(CAP))
+    k_knn_host_batch(Grid g, const ScanDesc* __restrict__ scans, int nscans, int64_t total_tiles, int tile, TileArgs a,
+                     float rho0) {
+    const int64_t item = work_item<CAP>(total_tiles, a.last_first);
+    if (item < 0) return;
+    const ScanDesc sd = scans[scan_of_item(scans, nscans, item)];
+    const int64_t n0 = (item - sd.tile0) * tile;
+    host_tile<CAP, G, COV, WIN>(g, sd.q, n0, (int)min((int64_t)tile, sd.n - n0), a, rho0, sd.idx, sd.d2, sd.cov);
+}
+
 __global__ void k_cov(Grid g, const int32_t* __restrict__ idx, int64_t N, int k, float eps,
                       float* __restrict__ cov) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1499,7 +1572,8 @@ __global__ void k_cov(Grid g, const int32_t* __restrict__ idx, int64_t N, int k,
     cov_row(g, idx + n * k, 1, k, eps, cov + 6 * n, true);
 }
 
-// The search kernel of FORM (0 one scan, 1 batched, 2 union) and WIN for mode
+// The search kernel of FORM (0 one scan, 1 batched, 2 union; 3 and 4: one scan
+// and batched into host memory, groups only) and WIN for mode
 // = search_mode(k) and `group` lanes per query of the group search; cov 0 none,
 // 1 plain, 2 weighted by a kernel descriptor.  (Weighted covariances have
 // kernels of their own: the descriptors' code beside the plain sums cost the
@@ -1508,7 +1582,9 @@ template <int FORM, bool WIN, int CAP, int G, int COV>
 void* form_kernel() {
     if constexpr (FORM == 0) return (void*)k_knn<CAP, G, COV, WIN>;
     else if constexpr (FORM == 1) return (void*)k_knn_batch<CAP, G, COV, WIN>;
-    else return (void*)k_knn_union<CAP, G, COV, WIN>;
+    else if constexpr (FORM == 2) return (void*)k_knn_union<CAP, G, COV, WIN>;
+    else if constexpr (FORM == 3) return (void*)k_knn_host<CAP, G, COV, WIN>;
+    else return (void*)k_knn_host_batch<CAP, G, COV, WIN>;
 }
 template <int FORM, bool WIN, int CAP, int G>
 void* form_kernel(int cov) {
@@ -1522,7 +1598,8 @@ void* form_kernel(int cov, int group) {
 }
 template <int FORM, bool WIN>
 void* knn_kernel(int mode, int cov, int group) {
-    if (mode == 2) return form_kernel<FORM, WIN, 0, 1>(cov);
+    if constexpr (FORM < 3)
+        if (mode == 2) return form_kernel<FORM, WIN, 0, 1>(cov);
     return mode == 0 ? form_kernel<FORM, WIN, 32>(cov, group) : form_kernel<FORM, WIN, 64>(cov, group);
 }
 

@@ -191,8 +191,8 @@ static pc_status build_target_internal(const float* xyz, int64_t M, const pc_bui
 // The search over the target as it stands: its grid, or its grid and the
 // delta grid of appended points searched as one map.
 static pc_status launch_search(pc_target_s* t, const float* q, int64_t N, int k, float eps, int32_t* idx,
-                               float* d2, float* cov, cudaStream_t st, bool host_cov = false) {
-    return pc_from_cuda(pc_launch_knn(t, q, N, k, eps, idx, d2, cov, pc_rho0(t, k), st, host_cov));
+                               float* d2, float* cov, cudaStream_t st, bool host_out = false) {
+    return pc_from_cuda(pc_launch_knn(t, q, N, k, eps, idx, d2, cov, pc_rho0(t, k), st, host_out));
 }
 
 // The device address of page-locked host memory mapped into the device's
@@ -482,7 +482,7 @@ pc_status pc_batch_plan(pc_target t, const pc_scan* scans, int n_scans, int k, f
     b->k = k;
     b->eps = eps;
     b->with_cov = sh.any_cov;
-    b->host_cov = sh.host_cov;
+    b->host_out = sh.host_out;
     b->tile = sh.tile;
     b->warps = sh.warps;
     b->total_tiles = sh.tiles;
@@ -512,7 +512,7 @@ pc_status pc_batch_run(pc_batch b, pc_stream s) {
     if (st == nullptr)  // the legacy stream cannot be captured: launch directly
         return pc_from_cuda(pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans,
                                                 b->total_tiles, b->total_queries, b->tile, b->warps, b->k, b->eps,
-                                                b->with_cov, b->host_cov, rho0, st));
+                                                b->with_cov, b->host_out, rho0, st));
     if (!b->exec || b->captured_on != st) {
         if (b->exec) cudaGraphExecDestroy(b->exec);
         if (b->graph) cudaGraphDestroy(b->graph);
@@ -522,7 +522,7 @@ pc_status pc_batch_run(pc_batch b, pc_stream s) {
         if (e != cudaSuccess) return pc_from_cuda(e);
         cudaError_t e2 = pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans, b->total_tiles,
                                              b->total_queries, b->tile, b->warps, b->k, b->eps, b->with_cov,
-                                             b->host_cov, rho0, st);
+                                             b->host_out, rho0, st);
         e = cudaStreamEndCapture(st, &b->graph);
         if (e2 != cudaSuccess) e = e2;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
@@ -551,12 +551,9 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
     if (t->delta) return PC_ERR_INVALID_ARG;  // appended points: pc_target_compact first
     if ((int64_t)k > t->g.m) return PC_ERR_K_GT_M;
     BatchShape sh;
-    sh.queries = 0;
-    for (int i = 0; i < n_scans; ++i) sh.queries += std::max<int64_t>(scans[i].n, 0);
-    sh.tile = pc_search_tile(t, k, sh.queries);
+    sh.queries = sh.tiles = 0;
     sh.warps = std::min(std::max(t->tune.warps, 1), 8);
-    sh.tiles = 0;
-    sh.any_cov = sh.host_cov = false;
+    sh.any_cov = sh.host_out = false;
     for (int i = 0; i < n_scans; ++i) {
         const pc_scan& sc = scans[i];
         if (sc.n < 0) return PC_ERR_INVALID_ARG;
@@ -565,11 +562,11 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
         if (sc.n > 0) {
             if (!sc.q_dev || !sc.idx_dev || !sc.d2_dev) return PC_ERR_INVALID_ARG;
             q = device_view(sc.q_dev);
-            idx = device_view(sc.idx_dev);
-            d2 = device_view(sc.d2_dev);
+            idx = device_view(sc.idx_dev, &sh.host_out);
+            d2 = device_view(sc.d2_dev, &sh.host_out);
             if (!q || !idx || !d2) return PC_ERR_BAD_POINTER;
             if (sc.cov_dev) {
-                if (!(cov = device_view(sc.cov_dev, &sh.host_cov))) return PC_ERR_BAD_POINTER;
+                if (!(cov = device_view(sc.cov_dev, &sh.host_out))) return PC_ERR_BAD_POINTER;
                 sh.any_cov = true;
             }
         }
@@ -578,8 +575,12 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
         table[i].idx = static_cast<int32_t*>(idx);
         table[i].d2 = static_cast<float*>(d2);
         table[i].cov = static_cast<float*>(cov);
+        sh.queries += sc.n;
+    }
+    sh.tile = pc_search_tile(t, k, sh.queries, sh.host_out);
+    for (int i = 0; i < n_scans; ++i) {
         table[i].tile0 = sh.tiles;
-        sh.tiles += (sc.n + sh.tile - 1) / sh.tile;
+        sh.tiles += (table[i].n + sh.tile - 1) / sh.tile;
     }
     *shape = sh;
     return PC_OK;
@@ -612,7 +613,7 @@ pc_status pc_batch_run_scratch(pc_target t, const pc_scan* scans, int n_scans, i
                                     cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = pc_launch_knn_batch(t, t->g, t->ck, table, n_scans, sh.tiles, sh.queries, sh.tile, sh.warps, k, eps,
-                                sh.any_cov, sh.host_cov, pc_rho0(t, k), st);
+                                sh.any_cov, sh.host_out, pc_rho0(t, k), st);
     return pc_from_cuda(e);
 }
 
