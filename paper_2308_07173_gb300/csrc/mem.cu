@@ -117,6 +117,10 @@ void pc_dev_free_idle(void* fence, void* const* ptrs, int n) {
         if (p->pool) cudaFreeAsync(ptrs[i], p->frees);
         else cudaFree(ptrs[i]);
     }
-    // the pool gives back what is above POOL_KEEP at a synchronisation
-    if (p->pool) cudaStreamSynchronize(p->frees);
+    // The pool gives back what is above POOL_KEEP at a synchronisation, asked for
+    // only then: on every close it cost the build of a 131k scan after it 45 us.
+    uint64_t held = 0;
+    if (p->pool && (cudaMemPoolGetAttribute(p->pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+                    held > POOL_KEEP))
+        cudaStreamSynchronize(p->frees);
 }
