@@ -334,13 +334,14 @@ __device__ __forceinline__ void scan_warp_box(const Grid& g, float qx, float qy,
 // g and the appended-points grid dg, whose point j is g.m + j: every
 // attempt scans both grids' boxes of the same radius, filtered by the
 // smaller of their two certified taus (a point of either grid outside its
-// box lies beyond both), and the exhaustive scan covers both grids.  The first
-// `fixed` attempts are those of a group search under a limit (above), from rho;
-// the widening proper then starts from rho1.
+// box lies beyond both), and the exhaustive scan covers both grids.  FIXED: the
+// first attempts are those of a group search under a limit (above), from rho,
+// and the widening proper starts from rho1.
 constexpr int SEARCH_OK = 0, SEARCH_LIMIT = 1, SEARCH_SHORT = 2;
-template <int SLOTS, bool DEL>
+template <int SLOTS, bool DEL, bool FIXED = false>
 __device__ int knn_search(const Grid& g, const Grid& dg, float qx, float qy, float qz, int k, float& rho,
-                          SearchState<SLOTS>& S, u64* pend, int lane, int fixed = 0, float rho1 = 0.0f) {
+                          SearchState<SLOTS>& S, u64* pend, int lane, float rho1 = 0.0f) {
+    int fixed = FIXED ? LIMITED_RADII : 0;
     for (int attempt = 0; attempt < 40 + LIMITED_RADII; ++attempt) {
         const WarpBox b = warp_box(g, qx, qy, qz, rho);
         WarpBox d = b;

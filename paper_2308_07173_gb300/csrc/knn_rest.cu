@@ -97,8 +97,9 @@ __device__ __forceinline__ void rest_body(const Grid& g, const Grid& dg, int64_t
                     rho = LIMITED_START * probe_radius<32, true>(g, true, qx, qy, qz, k, a.probe_c, lane);
                 SearchState<1> S;
                 state_reset(S);
-                const int sr = knn_search<1, DEL>(g, dg, qx, qy, qz, k, rho, S, s_pend[warp], lane,
-                                                  g.exhaustive ? 0 : LIMITED_RADII, rho1);
+                const int sr = g.exhaustive
+                                   ? knn_search<1, DEL>(g, dg, qx, qy, qz, k, rho, S, s_pend[warp], lane)
+                                   : knn_search<1, DEL, true>(g, dg, qx, qy, qz, k, rho, S, s_pend[warp], lane, rho1);
                 const bool ok = sr == SEARCH_OK;
                 if (!ok && lane == 0) atomicOr(g.status, sr == SEARCH_SHORT ? ST_SHORT : ST_SEARCH_LIMIT);
                 if (lane < k) {
