@@ -92,12 +92,14 @@ SPACE = {"occupancy": (8.0, 12.0, 16.0, 24.0), "rho_scale": (0.8, 0.9, 1.0), "wa
 
 
 def swept(k: int, space: Optional[dict] = None) -> dict:
-    """The parameters of `space` (SPACE by default) that reach a launch at this k: a group search (k <= 32) has
-    one-warp blocks and units of its own size, a warp search no survivor slots and no per-query radius.  Timing the
-    others would let noise pick a value."""
-    space = dict(SPACE if space is None else space)
-    for name in ("tile", "warps") if k <= 32 else ("slots", "probe"):
-        space.pop(name, None)
+    """What the descent sweeps at this k: the caller's space, or the parameters of SPACE that reach a launch.  A group
+    search (k <= 32) has one-warp blocks and units of its own size, a warp search no survivor slots and no per-query
+    radius; timing those would let noise pick a value."""
+    default = space is None
+    space = dict(SPACE if default else space)
+    if default:
+        for name in ("tile", "warps") if k <= 32 else ("slots", "probe"):
+            space.pop(name, None)
     if k > 24:
         space.pop("slots", None)  # 64 slots already
     return space
@@ -106,7 +108,7 @@ def swept(k: int, space: Optional[dict] = None) -> dict:
 def tune(map_xyz, queries, k: int, eps: float, space: Optional[dict] = None, rounds: int = 2, reps: int = 15,
          cache: Optional[str] = None, start: Optional[dict] = None) -> dict:
     """Coordinate descent over `space` (parameter -> values; SPACE by
-    default; those without effect at this k are left out) on (map_xyz [M,3], queries [N,3]) CUDA float32 tensors, from
+    default, without those that have no effect at this k) on (map_xyz [M,3], queries [N,3]) CUDA float32 tensors, from
     `start` (a configuration, e.g. an earlier best; DEFAULT otherwise);
     returns the best configuration (with its time in ms and cell size) and
     every configuration timed, and stores the best in `cache` if given."""

@@ -14,5 +14,4 @@ from paper_2308_07173_gb300 import autotune
 def test_swept_parameters(k, names):
     assert set(autotune.swept(k)) == names
     given = {"tile": (16, 32), "warps": (4,), "occupancy": (12.0,)}
-    assert set(autotune.swept(k, given)) == names & set(given)
-    assert set(given) == {"tile", "warps", "occupancy"}
+    assert autotune.swept(k, given) == given
