@@ -61,6 +61,12 @@ __device__ __forceinline__ float box_eta(const Grid& g, float px, float py, floa
 // linear scan of the whole map (exhaustive) or in `limited` with no pair.
 __device__ int nearest_within(const Grid& g, float px, float py, float pz, float max_d2, float r, float r1,
                               float& bd2, bool& limited) {
+    // nothing beyond max_dist can pair: a box of this half-width (max_dist and the
+    // margins of certified_tau) settles the point
+    const float pm = fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz)));
+    const float r_max = sqrtf(max_d2) * (1.0f + 0x1p-12f) + 0x1p-18f * (g.coord_scale + pm);
+    r = fminf(r, r_max);
+    float seen = 0.0f;  // no point within it
     for (int attempt = 0; attempt < 96; ++attempt) {
         const int ulx = cell_of(__fsub_rn(px, r), g.ox, g.inv_h);
         const int uhx = cell_of(__fadd_rn(px, r), g.ox, g.inv_h);
@@ -75,6 +81,7 @@ __device__ int nearest_within(const Grid& g, float px, float py, float pz, float
         const int64_t ncl = (int64_t)max(hx - lx + 1, 0) * max(hy - ly + 1, 0) * max(hz - lz + 1, 0);
         if (ncl > (int64_t)g.max_box_cells) {
             if (!(r1 > 0.0f)) break;
+            while (r1 <= seen) r1 *= 2.0f;
             r = r1;
             r1 = 0.0f;
             continue;
@@ -101,8 +108,9 @@ __device__ int nearest_within(const Grid& g, float px, float py, float pz, float
                 return (int)bpos;
             }
             if (tau >= max_d2) return -1;
+            seen = r;
         }
-        r = fminf(r * 2.0f, 1e30f);
+        r = r < r_max ? fminf(r * 2.0f, r_max) : fminf(r * 2.0f, 1e30f);
     }
     if (!g.exhaustive) {
         limited = true;
