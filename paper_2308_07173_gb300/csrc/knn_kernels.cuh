@@ -310,10 +310,10 @@ __device__ __forceinline__ bool group_allowed(const Grid& g, int64_t ncl, int64_
 }
 
 // Where the exact scan may not follow (exhaustive = 0), the radii decide which
-// queries are answered, so they do not follow the counts found: the group
-// search has LIMITED_RADII of them, LIMITED_START times the calibrated radius
-// and LIMITED_STEP times the one before, and k_knn_rest tries the same ones for
-// whatever a group could not sort before it widens up to max_box_cells.
+// queries are answered.  Those of a group search follow the counts it finds, so
+// for the queries it leaves k_knn_rest has LIMITED_RADII fixed ones, in boxes as
+// large as a group's: LIMITED_START times the calibrated radius, LIMITED_STEP
+// times the one before.  Then it widens from LIMITED_START up to max_box_cells.
 constexpr int LIMITED_RADII = 3;
 constexpr float LIMITED_START = 1.46f, LIMITED_STEP = 1.8f;
 
@@ -335,8 +335,8 @@ __device__ __forceinline__ void scan_warp_box(const Grid& g, float qx, float qy,
 // attempt scans both grids' boxes of the same radius, filtered by the
 // smaller of their two certified taus (a point of either grid outside its
 // box lies beyond both), and the exhaustive scan covers both grids.  FIXED: the
-// first attempts are those of a group search under a limit (above), from rho,
-// and the widening proper starts from rho1.
+// first attempts have the fixed radii above, from rho, and the widening proper
+// starts from rho1.
 constexpr int SEARCH_OK = 0, SEARCH_LIMIT = 1, SEARCH_SHORT = 2;
 template <int SLOTS, bool DEL, bool FIXED = false>
 __device__ int knn_search(const Grid& g, const Grid& dg, float qx, float qy, float qz, int k, float& rho,
@@ -775,7 +775,6 @@ __device__ void cov_row_any(const Grid& g, const Grid& dg, const int32_t* nb, in
 // registers and ran 1.35 waves of long warps.
 constexpr int MAX_ATTEMPTS = 6;
 constexpr float START = 1.4f;  // first radius over the calibrated starting radius; 1.26 and 1.54: 8 and 12 % slower
-__device__ __forceinline__ float start_factor(const Grid& g) { return g.exhaustive ? START : LIMITED_START; }
 constexpr int BATCH = 2;       // point loads a lane has in flight; 1 and 3: 3 % slower on scans
 constexpr uint32_t UNANSWERED = 0xffffffffu, UNIT_FLAG = 0x80000000u;
 constexpr uint32_t NAN_ROW = 0x7fc00000u;  // every entry of a covariance row without a value
@@ -1118,12 +1117,12 @@ __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const 
     {
         float r = rho0;
         if (a.probe_c > 0.0f) r = probe_radius<G, WIN>(g, finite, qx, qy, qz, k, a.probe_c, sub);
-        r *= start_factor(g);
+        r *= START;
         r2 = fminf(r * r, 1e30f);
     }
     float lo2 = 0.0f, hi2 = -1.0f;  // squared radii known to hold too few / too many (hi2 > 0)
     bool todo = finite, ok = false;
-    int w = 0, m = 0, wider = 0;
+    int w = 0, m = 0;
     float t = -1.0f;
     for (int attempt = 0; attempt < MAX_ATTEMPTS; ++attempt) {
         if (!__any_sync(FULL, todo)) break;
@@ -1166,11 +1165,7 @@ __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const 
         if (todo) {
             if (mm < (uint32_t)k) {  // widen; a wider box also certifies further
                 lo2 = r2;
-                float f = fminf(fmaxf(1.7f * (float)k / (float)max(mm, 1u), 1.5f), 9.0f);
-                if (!g.exhaustive) {
-                    f = LIMITED_STEP * LIMITED_STEP;
-                    if (!(hi2 > 0.0f) && ++wider == LIMITED_RADII) todo = false;
-                }
+                const float f = fminf(fmaxf(1.7f * (float)k / (float)max(mm, 1u), 1.5f), 9.0f);
                 r2 = hi2 > 0.0f ? 0.5f * (lo2 + hi2) : fminf(fmaxf(r2, 1e-6f * g.h * g.h) * f, 1e30f);
             } else if (over) {  // narrow
                 hi2 = tt;

@@ -91,7 +91,7 @@ __device__ __forceinline__ void rest_body(const Grid& g, const Grid& dg, int64_t
                     continue;
                 }
                 const float qx = __ldg(r.q + 3 * n), qy = __ldg(r.q + 3 * n + 1), qz = __ldg(r.q + 3 * n + 2);
-                const float rho1 = rho0 * start_factor(g);
+                const float rho1 = rho0 * (g.exhaustive ? START : LIMITED_START);
                 float rho = rho1;
                 if (!g.exhaustive && a.probe_c > 0.0f)
                     rho = LIMITED_START * probe_radius<32, true>(g, true, qx, qy, qz, k, a.probe_c, lane);
