@@ -45,7 +45,10 @@ int clamp_warps(int w) { return w <= 0 ? 4 : (w > 8 ? 8 : w); }
 // 42 / 33, 51 / 55; uniform box, k = 20 46 / 34, 53 / 50, 78 / 80.
 int group_lanes(int64_t n) { return n <= 24576 ? 8 : 4; }
 
-// form 0 one scan, 1 batched, 2 union, 3 and 4 one scan and batched into host memory
+// The forms of pc_internal.h, as one scan (0) or batched (1) and where the outputs lie.
+int host_form(int form, Out out, int mode) {
+    return mode == 2 || out == Out::device ? form : form + (out == Out::host_ragged ? 3 : 5);
+}
 void* search_kernel(int form, bool windowed, int mode, int cov, int group) {
     if (form >= 3)
         return windowed ? pc_knn_kernel_host_win(form, mode, cov, group) : pc_knn_kernel_host(form, mode, cov, group);
@@ -61,18 +64,18 @@ void* search_kernel(int form, bool windowed, int mode, int cov, int group) {
 cudaError_t launch_form(int form, const Grid& g, int mode, int cov, int64_t tiles, int tile, int warps, int k,
                         void** args, cudaStream_t s) {
     if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
-    const bool host = form >= 3;
-    const int group = mode < 2 ? 32 * (host ? HOST_WARPS : 1) / tile : 1;
+    const bool blocks = form == 3 || form == 4;
+    const int group = mode < 2 ? 32 * (blocks ? HOST_WARPS : 1) / tile : 1;
     void* kern = search_kernel(form, g.windowed != 0, mode, cov, group);
-    const int items = mode < 2 ? 1 : warps, threads = 32 * (mode == 2 ? warps : host ? HOST_WARPS : 1);
+    const int items = mode < 2 ? 1 : warps, threads = 32 * (mode == 2 ? warps : blocks ? HOST_WARPS : 1);
     return cudaLaunchKernel(kern, dim3((unsigned)((tiles + items - 1) / items)), dim3(threads), args,
-                            host ? host_stage_bytes(tile, k) : 0, s);
+                            blocks ? host_stage_bytes(tile, k) : 0, s);
 }
 
 int cov_kind(bool with_cov, const CovKernel& ck) { return !with_cov ? 0 : (ck.type == 0 ? 1 : 2); }
 
-TileArgs tile_args(const pc_target_s* t, const CovKernel& ck, int k, float eps, bool host) {
-    return TileArgs{k, eps, t->tune.order == 0 ? 1 : 0, ck, host ? 1 : 0, pc_probe_c(t)};
+TileArgs tile_args(const pc_target_s* t, const CovKernel& ck, int k, float eps, Out out) {
+    return TileArgs{k, eps, t->tune.order == 0 ? 1 : 0, ck, out == Out::device ? 0 : 1, pc_probe_c(t)};
 }
 
 }  // namespace
@@ -89,7 +92,7 @@ cudaError_t pc_knn_prepare() {
     std::lock_guard<std::mutex> lk(mu);
     if (done >> dev & 1) return cudaSuccess;
     cudaFuncAttributes at;
-    for (int form = 0; form < 5; ++form)
+    for (int form = 0; form < 7; ++form)
         for (int win = 0; win < 2; ++win)
             for (int mode = 0; mode < (form < 3 ? 3 : 2); ++mode)
                 for (int cov = 0; cov < (mode == 2 ? 2 : 3); ++cov)
@@ -104,8 +107,8 @@ cudaError_t pc_knn_prepare() {
 
 constexpr int64_t WARP_PATH_WARPS = 152 * 32;
 
-int pc_search_tile(const pc_target_s* t, int k, int64_t n, bool host_out) {
-    if (target_mode(t, k) < 2) return 32 * (host_out ? HOST_WARPS : 1) / group_lanes(n);
+int pc_search_tile(const pc_target_s* t, int k, int64_t n, Out out) {
+    if (target_mode(t, k) < 2) return 32 * (out == Out::host_ragged ? HOST_WARPS : 1) / group_lanes(n);
     // The warp path answers a tile's queries one after another on one warp
     // (each starts from the last one's radius): tiles shrink until a call has
     // as many warps as the chip holds at its 64 registers.  20k queries, k = 48
@@ -123,13 +126,12 @@ int pc_search_tile(const pc_target_s* t, int k, int64_t n, bool host_out) {
 // grid are searched as one map.
 cudaError_t pc_launch_knn(const pc_target_s* t, const float* q, int64_t N, int k, float eps,
                           int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s,
-                          bool host_out) {
+                          Out out) {
     if (N == 0) return cudaSuccess;
     const int mode = target_mode(t, k), warps = clamp_warps(t->tune.warps);
-    const bool host = host_out && mode < 2 && !t->delta;
-    const int tile = pc_search_tile(t, k, N, host);
+    const int tile = pc_search_tile(t, k, N, out);
     const int64_t tiles = (N + tile - 1) / tile;
-    TileArgs a = tile_args(t, t->ck, k, eps, host);
+    TileArgs a = tile_args(t, t->ck, k, eps, out);
     Grid g = t->g, dg = t->delta ? t->delta->g : t->g;
     cudaError_t e;
     if (t->delta) {
@@ -137,7 +139,7 @@ cudaError_t pc_launch_knn(const pc_target_s* t, const float* q, int64_t N, int k
         e = launch_form(2, g, mode, cov_kind(cov != nullptr, t->ck), tiles, tile, warps, k, args, s);
     } else {
         void* args[] = {&g, (void*)&q, (void*)&N, (void*)&tile, &a, &rho0, &idx, &d2, &cov};
-        e = launch_form(host ? 3 : 0, g, mode, cov_kind(cov != nullptr, t->ck), tiles, tile, warps, k, args, s);
+        e = launch_form(host_form(0, out, mode), g, mode, cov_kind(cov != nullptr, t->ck), tiles, tile, warps, k, args, s);
     }
     if (e != cudaSuccess || mode == 2) return e;
     return pc_launch_rest(g, t->delta ? &dg : nullptr, q, N, tile, a, rho0, idx, d2, cov, s);
@@ -154,16 +156,15 @@ cudaError_t pc_launch_cov(const pc_target_s* t, const int32_t* idx, int64_t N, i
 
 cudaError_t pc_launch_knn_batch(const pc_target_s* t, const Grid& gv, const CovKernel& ck,
                                 const ScanDesc* scans_dev, int nscans, int64_t total_tiles, int64_t queries,
-                                int tile, int warps, int k, float eps, bool with_cov, bool host_out, float rho0,
+                                int tile, int warps, int k, float eps, bool with_cov, Out out, float rho0,
                                 cudaStream_t s) {
     if (total_tiles == 0) return cudaSuccess;
     const int mode = target_mode(t, k);
-    const bool host = host_out && mode < 2;
-    TileArgs a = tile_args(t, ck, k, eps, host);
+    TileArgs a = tile_args(t, ck, k, eps, out);
     Grid g = gv;
     void* args[] = {&g, (void*)&scans_dev, &nscans, &total_tiles, &tile, &a, &rho0};
     const cudaError_t e =
-        launch_form(host ? 4 : 1, g, mode, cov_kind(with_cov, ck), total_tiles, tile, warps, k, args, s);
+        launch_form(host_form(1, out, mode), g, mode, cov_kind(with_cov, ck), total_tiles, tile, warps, k, args, s);
     if (e != cudaSuccess || mode == 2) return e;
     return pc_launch_rest_batch(g, scans_dev, nscans, total_tiles, queries, tile, a, rho0, s);
 }

@@ -773,8 +773,8 @@ __device__ void cov_row_any(const Grid& g, const Grid& dg, const int32_t* nb, in
 //    within 2^(TB-1) ulps; a group that finds two neighbours in one such
 //    bucket is put in exact (d2, index) order by an insertion sort.
 // 4. Rows are written by the warp as one contiguous block; three lanes of
-//    the group carry the covariance sums.  (Into host memory, by a block of
-//    four warps: k_knn_host.)
+//    the group carry the covariance sums.  (Into host memory off 128-byte
+//    lines, by a block of four warps: k_knn_host.)
 //
 // k_knn_rest follows every launch.  It turns the covariances into normals and
 // C' (eps >= 0), one query per lane, and answers the queries that no attempt
@@ -1095,10 +1095,11 @@ __device__ __forceinline__ float group_moments(float* c, const TileArgs& a, floa
 // the union of the main grid g and the grid dg of appended points (point j of
 // dg is g.m + j): both grids' boxes are walked, filtered by the smaller of
 // their certified taus, and list entries from dg carry DTAG.  idx, d2 and cov
-// point at the unit's own rows.  HOST: they are in shared memory, the
-// covariances are finished here and the caller sets the mark; returns whether
-// the unit has queries left for k_knn_rest.
-template <int CAP, int G, int COV, bool WIN, bool DEL, bool HOST = false>
+// point at the unit's own rows in device memory (HOST = 0), in mapped host memory
+// (1: covariances are finished here) or in shared memory on their way there (2:
+// so are they, and the caller sets the mark).  Returns whether the unit has
+// queries left for k_knn_rest.
+template <int CAP, int G, int COV, bool WIN, bool DEL, int HOST>
 __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const float* __restrict__ q, int cnt,
                                            const TileArgs& a, float rho0, int32_t* __restrict__ idx,
                                            float* __restrict__ d2, float* __restrict__ cov, unsigned char* smem) {
@@ -1111,7 +1112,7 @@ __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const 
     // k_knn_rest may be set up while the last blocks run (it waits for them)
     cudaTriggerProgrammaticLaunchCompletion();
     const int k = a.k;
-    const int lane = HOST ? threadIdx.x & 31 : threadIdx.x, sub = lane & (G - 1);
+    const int lane = HOST == 2 ? threadIdx.x & 31 : threadIdx.x, sub = lane & (G - 1);
     float* const ld = reinterpret_cast<float*>(smem);
     uint32_t* const lp = reinterpret_cast<uint32_t*>(smem + SLOTS * 32 * 4);
     uint32_t* const kb = reinterpret_cast<uint32_t*>(smem + SLOTS * 32 * 8);
@@ -1343,7 +1344,7 @@ __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const 
                 } else if (finm >> (qe * G) & 1u) {
                     dv = UNANSWERED;
                 }
-                if (!HOST && e == 0 && badm) dv |= UNIT_FLAG;
+                if (HOST < 2 && e == 0 && badm) dv |= UNIT_FLAG;
                 idx[e] = iv;
                 d2b[e] = dv;
             }
@@ -1370,7 +1371,7 @@ __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const 
     if (with_cov) {
         float uu, uv;
         const float total = group_moments<CS, KMAX, G, COV == 2>(ld + qi, a, qx, qy, qz, sub, uu, uv);
-        float* const sc = HOST ? cov : reinterpret_cast<float*>(kb);  // the keys are done with
+        float* const sc = HOST == 2 ? cov : reinterpret_cast<float*>(kb);  // the keys are done with
         const bool some = ok && total > 0.0f && isfinite(total);
         const float nan = __uint_as_float(NAN_ROW);
         if (sub < 3) {  // xx, xy; yy, yz; zz, xz
@@ -1378,11 +1379,12 @@ __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const 
             sc[6 * qi + (sub == 0 ? 1 : sub == 1 ? 4 : 2)] = some ? uv : nan;
         }
         __syncwarp();
-        if constexpr (HOST) {
+        if constexpr (HOST > 0) {  // a kernel of its own: as a branch it cost calls into device memory 2 us in spills
             if (sub == 0 && some) cov_regularise(sc + 6 * qi, a.eps);
-        } else {
-            for (int i = lane; i < 6 * cnt; i += 32) cov[i] = sc[i];
+            __syncwarp();
         }
+        if constexpr (HOST < 2)
+            for (int i = lane; i < 6 * cnt; i += 32) cov[i] = sc[i];
     }
     return badm != 0u;
 }
@@ -1457,13 +1459,13 @@ __device__ __forceinline__ int scan_of_item(const ScanDesc* __restrict__ scans, 
     return lo;
 }
 
-template <int CAP, int G, int COV, bool WIN, bool DEL>
+template <int CAP, int G, int COV, bool WIN, bool DEL, int HOST = 0>
 __device__ __forceinline__ void process_tile(const Grid& g, const Grid& dg, const float* __restrict__ q, int64_t n0,
                                              int cnt, const TileArgs& a, float rho0, int32_t* __restrict__ idx,
                                              float* __restrict__ d2, float* __restrict__ cov) {
     if constexpr (CAP > 0) {
         __shared__ __align__(16) unsigned char smem[group_warp_smem(CAP, G)];
-        group_unit<CAP, G, COV, WIN, DEL>(g, dg, q + 3 * n0, cnt, a, rho0, idx + n0 * a.k, d2 + n0 * a.k,
+        group_unit<CAP, G, COV, WIN, DEL, HOST>(g, dg, q + 3 * n0, cnt, a, rho0, idx + n0 * a.k, d2 + n0 * a.k,
                                           cov ? cov + 6 * n0 : nullptr, smem);
     } else {
         __shared__ u64 pend[8][64];
@@ -1476,19 +1478,19 @@ __device__ __forceinline__ void process_tile(const Grid& g, const Grid& dg, cons
 constexpr int block_threads(int cap) { return cap ? 32 : 256; }
 constexpr int block_target(int cap) { return cap == 32 ? 32 : cap == 64 ? 24 : 1; }
 
-template <int CAP, int G, int COV, bool WIN>
+template <int CAP, int G, int COV, bool WIN, int HOST = 0>
 __global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
     k_knn(Grid g, const float* __restrict__ q, int64_t N, int tile, TileArgs a, float rho0, int32_t* __restrict__ idx,
           float* __restrict__ d2, float* __restrict__ cov) {
     const int64_t t = work_item<CAP>((N + tile - 1) / tile, a.last_first);
     if (t < 0) return;
     const int64_t n0 = t * tile;
-    process_tile<CAP, G, COV, WIN, false>(g, g, q, n0, (int)min((int64_t)tile, N - n0), a, rho0, idx, d2, cov);
+    process_tile<CAP, G, COV, WIN, false, HOST>(g, g, q, n0, (int)min((int64_t)tile, N - n0), a, rho0, idx, d2, cov);
 }
 
 // Batched form: work items are the (scan, tile) pairs of the scans'
 // prefix-summed tile table, found by a binary search over the table.
-template <int CAP, int G, int COV, bool WIN>
+template <int CAP, int G, int COV, bool WIN, int HOST = 0>
 __global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
     k_knn_batch(Grid g, const ScanDesc* __restrict__ scans, int nscans, int64_t total_tiles, int tile, TileArgs a,
                 float rho0) {
@@ -1496,8 +1498,8 @@ __global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
     if (item < 0) return;
     const ScanDesc sd = scans[scan_of_item(scans, nscans, item)];
     const int64_t n0 = (item - sd.tile0) * tile;
-    process_tile<CAP, G, COV, WIN, false>(g, g, sd.q, n0, (int)min((int64_t)tile, sd.n - n0), a, rho0, sd.idx, sd.d2,
-                                          sd.cov);
+    process_tile<CAP, G, COV, WIN, false, HOST>(g, g, sd.q, n0, (int)min((int64_t)tile, sd.n - n0), a, rho0, sd.idx,
+                                                sd.d2, sd.cov);
 }
 
 // Search over a map grown by appended points: the main grid g and the
@@ -1512,20 +1514,21 @@ __global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
     process_tile<CAP, G, COV, WIN, true>(g, dg, q, n0, (int)min((int64_t)tile, N - n0), a, rho0, idx, d2, cov);
 }
 
-// Outputs in mapped host memory (k <= 32).  A block of four warps answers
-// HOST_WARPS units (32 queries, or 16 with eight lanes each), stages their rows
-// in shared memory and writes each array's rows as one block of 16-byte
-// vectors where the row base allows it.  Bounded by the host link (186 GB/s of
-// plain copies), which wants wide stores and long blocks.  A step of 1.45M
-// points, k = 20, 184 bytes each, and saturated served throughput (three steps
-// in flight):
-//   one warp, 4-byte stores in blocks of 640 bytes   2126 us  126 GB/s  6.94e8 points/s
-//   one warp, 16-byte vectors                        1822     147       8.07e8
-//   two warps, blocks of 1280 bytes                  1712     156       8.64e8
-//   four warps, blocks of 2560 bytes                 1648     162       8.92e8
-// (Eight would not fit 48 KB.)  The block has one mark: k_knn_rest reads them
-// back over the link, and one per unit cost 2 %.  Normals on 8 of 32 lanes
-// cost nothing here.
+// Outputs in mapped host memory off 128-byte lines (k <= 32): scans packed one
+// after another, a slice of a larger array.  Bounded by the host link (186 GB/s
+// of plain copies).  A warp's own rows, stored 128 bytes at a time, run at its
+// rate where those are whole lines and far below where each one straddles two,
+// so there a block of four warps answers HOST_WARPS units (32 queries, or 16
+// with eight lanes each), stages their rows in shared memory and writes each
+// array's rows as one block of 16-byte vectors where the row base allows it,
+// with one mark (k_knn_rest reads them back over the link).  us for 1M queries,
+// 2M map, one scan starting on a line / one row after it, and 16 scans packed:
+//   k = 20: one-warp units 1052 / 1739, 1437; staged 1058 / 1172, 1126
+//   k = 10:                 794 / 1166, 1115;         777 /  994,  873
+//   k = 32:                1563 / 1654, 1639;        1583 / 1611, 1601
+// 131k queries, k = 20: 177 / 278, 232; 185 / 197, 186.  In a step of 1.45M
+// points, blocks of 640, 1280 and 2560 bytes (one, two, four warps) reach 147,
+// 156 and 162 GB/s; eight warps would not fit 48 KB.
 constexpr int HOST_WARPS = 4;
 __host__ __device__ constexpr size_t host_stage_bytes(int tile, int k) {
     return (size_t)tile * (2 * k + 6) * sizeof(uint32_t);
@@ -1550,7 +1553,7 @@ __device__ __forceinline__ void host_tile(const Grid& g, const float* __restrict
     const int w = threadIdx.x >> 5, k = a.k, first = w * WQ;
     uint32_t* const sd = stage + TILE * k;
     uint32_t* const sc = sd + TILE * k;
-    const bool left = group_unit<CAP, G, COV, WIN, false, true>(
+    const bool left = group_unit<CAP, G, COV, WIN, false, 2>(
         g, g, q + 3 * (n0 + first), min(max(cnt - first, 0), WQ), a, rho0, reinterpret_cast<int32_t*>(stage) + first * k,
         reinterpret_cast<float*>(sd) + first * k, cov ? reinterpret_cast<float*>(sc) + 6 * first : nullptr, smem[w]);
     if (__syncthreads_or(left) && threadIdx.x == 0) sd[0] |= UNIT_FLAG;  // copied by thread 0
@@ -1589,8 +1592,8 @@ __global__ void k_cov(Grid g, const int32_t* __restrict__ idx, int64_t N, int k,
     cov_row(g, idx + n * k, 1, k, eps, cov + 6 * n, true);
 }
 
-// The search kernel of FORM (0 one scan, 1 batched, 2 union; 3 and 4: one scan
-// and batched into host memory, groups only) and WIN for mode
+// The search kernel of FORM (0 one scan, 1 batched, 2 union; into host memory,
+// groups only: 3 and 4 ragged, 5 and 6 on lines) and WIN for mode
 // = search_mode(k) and `group` lanes per query of the group search; cov 0 none,
 // 1 plain, 2 weighted by a kernel descriptor.  (Weighted covariances have
 // kernels of their own: the descriptors' code beside the plain sums cost the
@@ -1601,11 +1604,13 @@ void* form_kernel() {
     else if constexpr (FORM == 1) return (void*)k_knn_batch<CAP, G, COV, WIN>;
     else if constexpr (FORM == 2) return (void*)k_knn_union<CAP, G, COV, WIN>;
     else if constexpr (FORM == 3) return (void*)k_knn_host<CAP, G, COV, WIN>;
-    else return (void*)k_knn_host_batch<CAP, G, COV, WIN>;
+    else if constexpr (FORM == 4) return (void*)k_knn_host_batch<CAP, G, COV, WIN>;
+    else if constexpr (FORM == 5) return (void*)k_knn<CAP, G, COV, WIN, 1>;
+    else return (void*)k_knn_batch<CAP, G, COV, WIN, 1>;
 }
 template <int FORM, bool WIN, int CAP, int G>
 void* form_kernel(int cov) {
-    if (cov == 0) return form_kernel<FORM, WIN, CAP, G, 0>();
+    if (cov == 0) return form_kernel<FORM < 5 ? FORM : FORM - 5, WIN, CAP, G, 0>();  // nothing to finish
     if (CAP == 0 || cov == 1) return form_kernel<FORM, WIN, CAP, G, 1>();
     return form_kernel<FORM, WIN, CAP, G, CAP == 0 ? 1 : 2>();
 }

@@ -8,15 +8,15 @@
 // other queries took 0.1 ms.
 //
 // Here every warp answers one query at a time.  A block reads the marks of
-// 32 work items (units of up to 8 queries; into host memory up to 32 queries
-// with one mark), strided by the grid so that neighbouring ones fall to
+// 32 work items (units of up to 8 queries; into ragged host memory up to
+// 32 queries with one mark), strided by the grid so that neighbouring ones fall to
 // different blocks, and its 8 warps take a marked item's rows.  The grid fills
 // the chip from 608 items on: leftovers, not marks, take the time (60k queries
 // around 40 tight clusters into host memory: 22.2 ms with a block per 32 items,
 // 5.6 with the staged search before groups, 3.6 now).
 //
 // First the block turns its units' covariances into C' = I - (1 - eps) n n^T
-// (eps >= 0; the search into host memory has done so), one query per lane.  Inside the search this ran on one warp of
+// (eps >= 0; done in the search into host memory), one query per lane.  Inside the search this ran on one warp of
 // a block while the others idled, or on 8 of 32 lanes: 10 of 73 us of the
 // 131k scan, k = 20.  Rows without a value (NAN_ROW) are left alone, among
 // them the unanswered ones, which get theirs complete.
@@ -44,7 +44,7 @@ __device__ __forceinline__ void rest_body(const Grid& g, const Grid& dg, int64_t
     __shared__ unsigned s_marked;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = a.k;
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&g.stats[0], (unsigned long long)queries);
-    const bool regularise = a.eps >= 0.0f && !a.host;
+    const bool regularise = a.eps >= 0.0f && !a.finish;
     cudaGridDependencySynchronize();  // the search's rows and marks are complete and visible
     for (int64_t base = blockIdx.x; base < tiles; base += (int64_t)32 * gridDim.x) {
         if (warp == 0) {

@@ -191,8 +191,8 @@ static pc_status build_target_internal(const float* xyz, int64_t M, const pc_bui
 // The search over the target as it stands: its grid, or its grid and the
 // delta grid of appended points searched as one map.
 static pc_status launch_search(pc_target_s* t, const float* q, int64_t N, int k, float eps, int32_t* idx,
-                               float* d2, float* cov, cudaStream_t st, bool host_out = false) {
-    return pc_from_cuda(pc_launch_knn(t, q, N, k, eps, idx, d2, cov, pc_rho0(t, k), st, host_out));
+                               float* d2, float* cov, cudaStream_t st, Out out = Out::device) {
+    return pc_from_cuda(pc_launch_knn(t, q, N, k, eps, idx, d2, cov, pc_rho0(t, k), st, out));
 }
 
 // The device address of page-locked host memory mapped into the device's
@@ -207,10 +207,16 @@ static void* mapped_host(const void* p) {
     return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+// Output p in mapped host memory, beside the others of a call.
+static Out host_out(const void* p, Out others = Out::device) {
+    return others == Out::host_ragged || (reinterpret_cast<uintptr_t>(p) & 127) != 0 ? Out::host_ragged
+                                                                                   : Out::host_lines;
+}
+
 // The address kernels use for p: p itself for device (or managed) memory,
-// the device address of mapped page-locked host memory (and *host = true),
+// the device address of mapped page-locked host memory (noted in *out),
 // null for anything else.
-static void* device_view(const void* p, bool* host = nullptr) {
+static void* device_view(const void* p, Out* out = nullptr) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
@@ -218,7 +224,7 @@ static void* device_view(const void* p, bool* host = nullptr) {
     }
     if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) return const_cast<void*>(p);
     if (a.type == cudaMemoryTypeHost && a.devicePointer) {
-        if (host) *host = true;
+        if (out) *out = host_out(a.devicePointer, *out);
         return a.devicePointer;
     }
     return nullptr;
@@ -407,7 +413,7 @@ pc_status pc_knn_cov_host(pc_target t, const float* q_host, int64_t N, int k, fl
             q = qs;
         }
         r = launch_search(t, q, N, k, eps, static_cast<int32_t*>(mi), static_cast<float*>(md),
-                          static_cast<float*>(mc), st, true);
+                          static_cast<float*>(mc), st, host_out(mc, host_out(md, host_out(mi))));
         if (r != PC_OK) return r;
         return read_and_clear_status(t, st);
     }
@@ -482,7 +488,7 @@ pc_status pc_batch_plan(pc_target t, const pc_scan* scans, int n_scans, int k, f
     b->k = k;
     b->eps = eps;
     b->with_cov = sh.any_cov;
-    b->host_out = sh.host_out;
+    b->out = sh.out;
     b->tile = sh.tile;
     b->warps = sh.warps;
     b->total_tiles = sh.tiles;
@@ -512,7 +518,7 @@ pc_status pc_batch_run(pc_batch b, pc_stream s) {
     if (st == nullptr)  // the legacy stream cannot be captured: launch directly
         return pc_from_cuda(pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans,
                                                 b->total_tiles, b->total_queries, b->tile, b->warps, b->k, b->eps,
-                                                b->with_cov, b->host_out, rho0, st));
+                                                b->with_cov, b->out, rho0, st));
     if (!b->exec || b->captured_on != st) {
         if (b->exec) cudaGraphExecDestroy(b->exec);
         if (b->graph) cudaGraphDestroy(b->graph);
@@ -522,7 +528,7 @@ pc_status pc_batch_run(pc_batch b, pc_stream s) {
         if (e != cudaSuccess) return pc_from_cuda(e);
         cudaError_t e2 = pc_launch_knn_batch(b->t, b->g, b->ck, b->scans_dev, b->n_scans, b->total_tiles,
                                              b->total_queries, b->tile, b->warps, b->k, b->eps, b->with_cov,
-                                             b->host_out, rho0, st);
+                                             b->out, rho0, st);
         e = cudaStreamEndCapture(st, &b->graph);
         if (e2 != cudaSuccess) e = e2;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
@@ -553,7 +559,8 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
     BatchShape sh;
     sh.queries = sh.tiles = 0;
     sh.warps = std::min(std::max(t->tune.warps, 1), 8);
-    sh.any_cov = sh.host_out = false;
+    sh.any_cov = false;
+    sh.out = Out::device;
     for (int i = 0; i < n_scans; ++i) {
         const pc_scan& sc = scans[i];
         if (sc.n < 0) return PC_ERR_INVALID_ARG;
@@ -562,11 +569,11 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
         if (sc.n > 0) {
             if (!sc.q_dev || !sc.idx_dev || !sc.d2_dev) return PC_ERR_INVALID_ARG;
             q = device_view(sc.q_dev);
-            idx = device_view(sc.idx_dev, &sh.host_out);
-            d2 = device_view(sc.d2_dev, &sh.host_out);
+            idx = device_view(sc.idx_dev, &sh.out);
+            d2 = device_view(sc.d2_dev, &sh.out);
             if (!q || !idx || !d2) return PC_ERR_BAD_POINTER;
             if (sc.cov_dev) {
-                if (!(cov = device_view(sc.cov_dev, &sh.host_out))) return PC_ERR_BAD_POINTER;
+                if (!(cov = device_view(sc.cov_dev, &sh.out))) return PC_ERR_BAD_POINTER;
                 sh.any_cov = true;
             }
         }
@@ -577,7 +584,7 @@ pc_status pc_batch_table(const pc_target_s* t, const pc_scan* scans, int n_scans
         table[i].cov = static_cast<float*>(cov);
         sh.queries += sc.n;
     }
-    sh.tile = pc_search_tile(t, k, sh.queries, sh.host_out);
+    sh.tile = pc_search_tile(t, k, sh.queries, sh.out);
     for (int i = 0; i < n_scans; ++i) {
         table[i].tile0 = sh.tiles;
         sh.tiles += (table[i].n + sh.tile - 1) / sh.tile;
@@ -613,7 +620,7 @@ pc_status pc_batch_run_scratch(pc_target t, const pc_scan* scans, int n_scans, i
                                     cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = pc_launch_knn_batch(t, t->g, t->ck, table, n_scans, sh.tiles, sh.queries, sh.tile, sh.warps, k, eps,
-                                sh.any_cov, sh.host_out, pc_rho0(t, k), st);
+                                sh.any_cov, sh.out, pc_rho0(t, k), st);
     return pc_from_cuda(e);
 }
 

@@ -21,13 +21,17 @@ struct CovKernel {
     float ox, oy, oz;
 };
 
+// Where a search's outputs lie: device memory, or mapped page-locked host memory
+// with every array on a 128-byte line, or off one.
+enum class Out { device, host_lines, host_ragged };
+
 // What a search launch passes to its kernels besides the grid and buffers.
 struct TileArgs {
     int k;
     float eps;
     int last_first;  // issue tiles from the end of the query array
     CovKernel ck;    // kernel-descriptor weights; type 0: the plain covariance
-    int host;        // group search into host memory: tiles of HOST_WARPS units, covariances finished in the search
+    int finish;      // group search: regularise in the search (outputs in host memory) instead of in k_knn_rest
     float probe_c;   // > 0: every query estimates its own starting radius (probe_radius)
 };
 
@@ -85,7 +89,7 @@ struct pc_batch_s {
     int k;
     float eps;
     bool with_cov;
-    bool host_out;  // some output is mapped host memory
+    Out out;
     int tile;
     int warps;
     int64_t total_tiles;
@@ -148,9 +152,9 @@ cudaError_t pc_scan_exclusive(const uint32_t* in, uint32_t* out, int64_t n, uint
                               uint32_t* temp, cudaStream_t s);
 
 // The search kernels' translation units (whole-map / window variants, with or
-// without appended points): form 0 one scan, 1 batched, 2 union, 3 and 4 one
-// scan and batched into host memory (k <= 32); group: lanes per query of the
-// group search (k <= 32).
+// without appended points): form 0 one scan, 1 batched, 2 union; k <= 32 into
+// host memory: 3 one scan and 4 batched, ragged, 5 and 6 the same on lines;
+// group: lanes per query of the group search (k <= 32).
 void* pc_knn_kernel_win(int form, int mode, int cov, int group);
 void* pc_knn_kernel_batch(int mode, int cov, int group);
 void* pc_knn_kernel_batch_win(int mode, int cov, int group);
@@ -159,21 +163,21 @@ void* pc_knn_kernel_union_win(int mode, int cov, int group);
 void* pc_knn_kernel_host(int host_form, int mode, int cov, int group);
 void* pc_knn_kernel_host_win(int host_form, int mode, int cov, int group);
 
-// knn_cov.cu.  host_out: the outputs are mapped page-locked host memory.
+// knn_cov.cu
 cudaError_t pc_launch_knn(const pc_target_s* t, const float* q, int64_t N, int k, float eps,
-                          int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s, bool host_out = false);
+                          int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s, Out out = Out::device);
 // Loads every search kernel on the current device (once; called by the first
 // build, so that no search or capture is the first to launch one).
 cudaError_t pc_knn_prepare();
 cudaError_t pc_rest_prepare();
 // Queries of one work item of a search over n queries (k <= 32: a unit of the
-// group search, or a block's units into host memory; else the tune's tile).
-int pc_search_tile(const pc_target_s* t, int k, int64_t n, bool host_out);
+// group search, or a block's units into ragged host memory; else the tune's tile).
+int pc_search_tile(const pc_target_s* t, int k, int64_t n, Out out);
 cudaError_t pc_launch_cov(const pc_target_s* t, const int32_t* idx, int64_t N, int k, float eps,
                           float* cov, cudaStream_t s);
 cudaError_t pc_launch_knn_batch(const pc_target_s* t, const pcdev::Grid& g, const CovKernel& ck,
                                 const ScanDesc* scans_dev, int nscans, int64_t total_tiles, int64_t queries,
-                                int tile, int warps, int k, float eps, bool with_cov, bool host_out, float rho0,
+                                int tile, int warps, int k, float eps, bool with_cov, Out out, float rho0,
                                 cudaStream_t s);
 
 // knn_rest.cu: the queries that a group search (k <= 32) over the same
@@ -207,7 +211,7 @@ struct BatchShape {
     int tile, warps;
     int64_t queries;
     bool any_cov;   // some scan asks for covariances
-    bool host_out;  // some output is mapped host memory
+    Out out;        // where some output lies that is not device memory
 };
 // Argument checks and scan table shared by pc_batch_plan,
 // pc_batch_run_scratch and pc_batch_run_noalloc; fills table[0, n_scans)

@@ -1,7 +1,7 @@
-"""Searches that write page-locked host memory (k <= 32): blocks of four units
-with remainders, rows that start off 16-byte boundaries, far, equal and
-non-finite queries in every place of a block, windows and weights.  Every row
-equals the device-memory search's bit for bit."""
+"""Searches that write page-locked host memory (k <= 32): rows on 128-byte lines
+(one-warp units) and off them (blocks of four units with remainders), far, equal
+and non-finite queries in every place of a block, windows and weights.  Every
+row equals the device-memory search's bit for bit."""
 import numpy as np
 import pytest
 
@@ -42,8 +42,8 @@ def test_rows_in_host_memory(gpu_lib, n, k, setting):
     for eps in (1e-3, -1.0):
         want = t.knn_cov(dev(q), k, eps)
         t.sync_status()
-        for off in (0, 1):  # rows from the array's start, and from its second row
-            out = tuple(torch.full((n + 1, w), -7, dtype=d, pin_memory=True)
+        for off in (0, 1, 32):  # rows from a line, from off one, and from a later line
+            out = tuple(torch.full((n + 33, w), -7, dtype=d, pin_memory=True)
                         for w, d in ((k, torch.int32), (k, torch.float32), (6, torch.float32)))
             part = tuple(o[off:off + n] for o in out)
             qp = torch.from_numpy(q).pin_memory()
@@ -52,13 +52,13 @@ def test_rows_in_host_memory(gpu_lib, n, k, setting):
             for a, b in zip(part, want):
                 assert torch.equal(bits(a), bits(b))
             for o in out:
-                assert (o[n if off == 0 else 0] == -7).all()  # nothing beside the rows
+                assert (o[:off] == -7).all() and (o[off + n:] == -7).all()  # nothing beside the rows
     t.close()
 
 
 @pytest.mark.parametrize("with_cov", [True, False])
 @pytest.mark.parametrize("k", [5, 20, 32])
-@pytest.mark.parametrize("sizes", [(1, 40, 0, 17), (31, 33, 9000, 5), (20_001, 8_000, 3)])
+@pytest.mark.parametrize("sizes", [(1, 40, 0, 17), (31, 33, 9000, 5), (20_001, 8_000, 3), (32, 640, 24_000, 7)])
 def test_batches_in_host_memory(gpu_lib, sizes, k, with_cov):
     n = sum(sizes)
     m, q = queries(n, n + k)
