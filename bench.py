@@ -756,18 +756,20 @@ def run_c5(args):
                      "warp_search_frac": st["warp_search"] / max(1, st["queries"]),
                      "exhaustive": st["exhaustive"], "candidates_per_query": st["candidates"] / max(1, st["queries"])}
     info = t.info()
-    best = out["per_query_start"]
+    start = "calibrated_start" if cfg["probe"] == 1 else "per_query_start"  # the tuned configuration's
+    best = out[start]
     roof = algorithmic_roofline(md, info, [idx], len(q), k, best["ms"])
     _line("query points/sec, 1M queries vs 20M-point map (4 km + pit lane), kNN(k=32)+cov",
           best["value"], UNIT, best["ms"], args,
           {"workload": "c5_map20M_pit_noise1cm_queries1M_k32", "queries": len(q), "map_points": len(m),
            "cell_size": info["cell_size"], "occupied_cells": info["ncells"],
            "tuned": tuned or "defaults (no cached configuration)",
-           "start_radius": "per query, from the point count of the 27 cells around it (the target's default "
-                           "on this map: its calibration saw an uneven density)"},
+           "start_radius": {"calibrated_start": "one calibrated radius for the map",
+                            "per_query_start": "per query, from the point count of the 27 cells around it"}[start]},
           roofline=roof, search_paths={"warp_search_frac": best["warp_search_frac"], "exhaustive": best["exhaustive"],
                                        "candidates_per_query": best["candidates_per_query"]},
-          clocks=best["clocks"], calibrated_start=out["calibrated_start"], gpu_launches=2)
+          clocks=best["clocks"], per_query_start=out["per_query_start"],
+          calibrated_start=out["calibrated_start"], gpu_launches=2)
     return 0
 
 
