@@ -192,11 +192,10 @@ __device__ __forceinline__ float cell_lower_bound2(const Grid& g, float qx, floa
 // box of half-width R cells costs ~(2R + 1) row lookups per level of z where
 // the hash costs (2R + 1)^2 cell probes, so the search can widen to any
 // distance; the per-row cut drops the rows that the k found so far exclude.
-// Measured (131k-point scan searched with itself, k = 20; the 700 to 1,000
-// queries in its sparse rim find their 20th neighbour up to 100 cells away
-// and, cell by cell, ended in the scan of every occupied cell): 9.8-36 ms
-// by cells, 0.73-0.89 ms by rows; k = 48, 20k queries of a 300k map, where
-// every query takes this search: 0.209 -> 0.188 ms.
+// Measured on a 131k-point scan searched with itself, k = 20, where the 700 to
+// 1,000 queries in its sparse rim find their 20th neighbour up to 100 cells away
+// and, cell by cell, ended in the scan of every occupied cell: 9.8-36 ms by
+// cells, 0.16-0.25 ms by rows from k_knn_rest.
 template <int SLOTS>
 __device__ void scan_rows(const Grid& g, float qx, float qy, float qz, int lx, int ly, int lz,
                           int ex, int ey, int ez, float eta, float tau, SearchState<SLOTS>& S, u64* pend,
@@ -1474,12 +1473,17 @@ __device__ __forceinline__ void process_tile(const Grid& g, const Grid& dg, cons
 }
 
 // Threads of a block and, for the group search, blocks an SM should hold: 32
-// one-warp blocks (64 registers, 5 KB each), 24 with 64 sorted survivors.
+// one-warp blocks (64 registers, 5 KB each), 24 (80 registers) with 64 sorted
+// survivors, and with eight lanes a query under a window, with weights or over
+// two grids, which spill up to 190 bytes at 64: calls of 300 to 4,000 queries,
+// k = 10 to 20, take 20-23 us with 64 and 18-21 with 80 registers (of 20,000, 29
+// and 27). The plain form does not spill and gains nothing.
 constexpr int block_threads(int cap) { return cap ? 32 : 256; }
-constexpr int block_target(int cap) { return cap == 32 ? 32 : cap == 64 ? 24 : 1; }
+constexpr int block_target(int cap, bool heavy) { return cap == 32 ? (heavy ? 24 : 32) : cap == 64 ? 24 : 1; }
+constexpr bool heavy_form(int g, int cov, bool win, bool del) { return g == 8 && (cov == 2 || win || del); }
 
 template <int CAP, int G, int COV, bool WIN, int HOST = 0>
-__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
+__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP, heavy_form(G, COV, WIN, false)))
     k_knn(Grid g, const float* __restrict__ q, int64_t N, int tile, TileArgs a, float rho0, int32_t* __restrict__ idx,
           float* __restrict__ d2, float* __restrict__ cov) {
     const int64_t t = work_item<CAP>((N + tile - 1) / tile, a.last_first);
@@ -1491,7 +1495,7 @@ __global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
 // Batched form: work items are the (scan, tile) pairs of the scans'
 // prefix-summed tile table, found by a binary search over the table.
 template <int CAP, int G, int COV, bool WIN, int HOST = 0>
-__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
+__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP, heavy_form(G, COV, WIN, false)))
     k_knn_batch(Grid g, const ScanDesc* __restrict__ scans, int nscans, int64_t total_tiles, int tile, TileArgs a,
                 float rho0) {
     const int64_t item = work_item<CAP>(total_tiles, a.last_first);
@@ -1505,7 +1509,7 @@ __global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
 // Search over a map grown by appended points: the main grid g and the
 // appended-points grid dg as one map (indices of dg's points follow g's).
 template <int CAP, int G, int COV, bool WIN>
-__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP))
+__global__ void __launch_bounds__(block_threads(CAP), block_target(CAP, heavy_form(G, COV, WIN, true)))
     k_knn_union(Grid g, Grid dg, const float* __restrict__ q, int64_t N, int tile, TileArgs a, float rho0,
                 int32_t* __restrict__ idx, float* __restrict__ d2, float* __restrict__ cov) {
     const int64_t t = work_item<CAP>((N + tile - 1) / tile, a.last_first);
