@@ -127,9 +127,10 @@ typedef struct {
 /* One scan of a batch, caller-owned: device memory, or page-locked host
  * memory mapped into the device's address space (cudaHostAlloc,
  * cudaHostRegister, torch pin_memory).  When any scan's idx, d2 or cov is
- * such host memory, each warp writes its queries' rows as whole blocks, so
- * the results reach host memory during the search with no copy (for k <= 32;
- * the warp path, k > 32, writes row by row).  Results are identical either way.  Any other pointer returns
+ * such host memory, rows leave in contiguous blocks, so the results reach host
+ * memory during the search with no copy (for k <= 32; the warp path, k > 32,
+ * writes row by row).  Fastest where idx, d2 and cov of every scan start on
+ * 128-byte lines.  Results are identical either way.  Any other pointer returns
  * PC_ERR_BAD_POINTER. */
 typedef struct {
     const float *q_dev; /* [n,3] */

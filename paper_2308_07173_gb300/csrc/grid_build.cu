@@ -577,8 +577,7 @@ cudaError_t radix_sort(u64*& keys, uint32_t*& vals, u64* keys_alt, uint32_t* val
 }  // namespace
 
 // Sort and scan on caller buffers (used by the wall detector, which sizes
-// everything once at creation).
-// for any count up to n
+// everything once at creation: the words of any count up to n).
 size_t pc_sort_temp_words(int64_t n) {
     const int64_t nb = std::max(rs_blocks(n), rs_blocks(std::min(n, RS_SMALL)));
     return (size_t)256 * (size_t)std::max<int64_t>(nb, 1) + 256;

@@ -105,14 +105,17 @@ cudaError_t pc_knn_prepare() {
     return cudaSuccess;
 }
 
+// 32 warps an SM, of which 20 are resident at once (the warp path takes 92
+// registers). 20k queries, k = 48 on a 300k map, with 20, 32, 48 warps an SM: 89,
+// 84, 96 us; 40k: 154, 138, 142; 131k: 417, 381, 368.
 constexpr int64_t WARP_PATH_WARPS = 152 * 32;
 
 int pc_search_tile(const pc_target_s* t, int k, int64_t n, Out out) {
     if (target_mode(t, k) < 2) return 32 * (out == Out::host_ragged ? HOST_WARPS : 1) / group_lanes(n);
     // The warp path answers a tile's queries one after another on one warp
     // (each starts from the last one's radius): tiles shrink until a call has
-    // as many warps as the chip holds at its 64 registers.  20k queries, k = 48
-    // on a 300k map, tiles of 32 (4 warps an SM): 188 us, of 4: 96 us.
+    // WARP_PATH_WARPS.  20k queries, k = 48 on a 300k map, tiles of 32 (4 warps an
+    // SM): 188 us, of 4: 84.
     // Not where the exact scan may not follow (exhaustive = 0): there the radius
     // a query starts from decides whether it is answered, and must not depend
     // on the size of the call.

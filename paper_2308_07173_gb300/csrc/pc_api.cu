@@ -154,7 +154,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 // Builds a target over xyz.  With `like` (the grid of appended points), the
 // cell edge and the starting radii are taken from that target instead of
 // the cell-size bisection and the calibration search: both grids are then
-// searched with one trial radius, and an append costs one grid build.
+// searched with one starting radius, and an append costs one grid build.
 static pc_status build_target_internal(const float* xyz, int64_t M, const pc_build_opts& o, cudaStream_t st,
                                        pc_target_s** out, const pc_target_s* like = nullptr) {
     if (capturing(st)) return PC_ERR_CUDA;
@@ -397,8 +397,8 @@ pc_status pc_knn_cov_host(pc_target t, const float* q_host, int64_t N, int k, fl
     DeviceGuard dg(t->device);
     cudaStream_t st = (cudaStream_t)s;
     // Page-locked outputs (k <= 32, no appended points): the search writes
-    // them in place, each warp's rows as one block, so the transfer runs
-    // during the search; a page-locked q is read in place too.  (The warp
+    // them in place, block by block, so the transfer runs during the search; a
+    // page-locked q is read in place too.  (The warp
     // path writes row by row, so wider k keeps the staged copies.)
     void* const mi = (k <= 32 && !t->delta) ? mapped_host(idx_host) : nullptr;
     void* const md = mi ? mapped_host(d2_host) : nullptr;

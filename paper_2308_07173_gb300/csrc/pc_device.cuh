@@ -54,7 +54,7 @@ struct Grid {
     const uint2* xcut;
     int* status;
     unsigned long long* stats;  // [0] queries, [1] warp-search fallbacks, [2] exhaustive scans,
-                                // [3] lane-path candidate points
+                                // [3] points the group search visited
     // Search window (pc_set_window): only target points p with
     // wlo <= p <= whi (componentwise) are searched.  [wl, wh] is the range of
     // cells that can hold them (the whole grid when windowed == 0); a point

@@ -203,7 +203,7 @@ cudaError_t pc_launch_pack_xyz(const pc_target_s* t, float* out, cudaStream_t s)
 
 // pc_api.cu
 float pc_rho0(const pc_target_s* t, int k);
-// The probe constant of the lane path's per-query starting radius (0: off).
+// The probe constant of the group search's per-query starting radius (0: off).
 float pc_probe_c(const pc_target_s* t);
 // Launch shape of a batched call over caller-provided scans.
 struct BatchShape {

@@ -20,8 +20,8 @@ GPU).  The map's grid stays resident on the device.  The loop:
   and kernel overlap the steps already on the GPU;
 * or, with ``in_place=True``, points the step's scan table at the requests'
   page-locked scans and the slot's page-locked outputs: the batched kernel
-  reads the scans and writes the results in host memory itself (each warp
-  its tile's rows as whole blocks), with no copies and no device buffers
+  reads the scans and writes the results in host memory itself, in
+  contiguous blocks of rows, with no copies and no device buffers
   beyond the scan table;
 * retires steps whose completion event has fired, frees their slot, and
   stamps each request's completion time.
