@@ -110,7 +110,7 @@ __device__ int nearest_within(const Grid& g, float px, float py, float pz, float
             if (tau >= max_d2) return -1;
             seen = r;
         }
-        r = r < r_max ? fminf(r * 2.0f, r_max) : fminf(r * 2.0f, 1e30f);
+        r = r < r_max ? fminf(r * 2.0f, r_max) : fminf(fmaxf(r, 0x1p-10f * g.h) * 2.0f, 1e30f);
     }
     if (!g.exhaustive) {
         limited = true;

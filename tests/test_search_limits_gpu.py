@@ -83,6 +83,20 @@ def test_gicp_reach(gpu_lib, cells):
     np.testing.assert_array_equal(corr[corr >= 0], oracle.knn_brute(src, mp, 1)[0][corr >= 0, 0])
 
 
+@pytest.mark.parametrize("max_dist", [0.0, 1e-30, 1e-3, 1.0])
+@pytest.mark.parametrize("exhaustive", [False, True])
+def test_gicp_max_dist_of_nothing(gpu_lib, exhaustive, max_dist):
+    """A map and a source of one place, the origin: no scale to take margins from."""
+    mp, src = np.zeros((5, 3), F), np.zeros((40, 3), F)
+    src[1::2, 0] = 2.0
+    t = gpu_lib.Target(dev(mp), exhaustive=exhaustive)
+    want = np.where(np.arange(40) % 2 == 0, 0, -1)
+    np.testing.assert_array_equal(pairs(t, mp, src, max_dist), want)
+    assert t.sync_status() == gpu_lib.PC_OK
+    assert t.stats()["exhaustive"] == 0
+    t.close()
+
+
 # ---------------------------------------------------------------- kNN
 @pytest.mark.parametrize("n", [3000, 24_600])
 @pytest.mark.parametrize("k", [1, 10, 20, 32])
