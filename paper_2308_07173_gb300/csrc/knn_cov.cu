@@ -131,6 +131,7 @@ cudaError_t pc_launch_knn(const pc_target_s* t, const float* q, int64_t N, int k
                           int32_t* idx, float* d2, float* cov, float rho0, cudaStream_t s,
                           Out out) {
     if (N == 0) return cudaSuccess;
+    if (t->delta) out = Out::device;  // the union search has no host forms; its rows may lie anywhere
     const int mode = target_mode(t, k), warps = clamp_warps(t->tune.warps);
     const int tile = pc_search_tile(t, k, N, out);
     const int64_t tiles = (N + tile - 1) / tile;

@@ -789,6 +789,7 @@ __device__ void cov_row_any(const Grid& g, const Grid& dg, const int32_t* nb, in
 // registers and ran 1.35 waves of long warps.
 constexpr int MAX_ATTEMPTS = 6;
 constexpr float START = 1.4f;  // first radius over the calibrated starting radius; 1.26 and 1.54: 8 and 12 % slower
+constexpr int64_t SMALL_MAP = 2048;  // points a group may well walk several times
 constexpr int BATCH = 2;       // point loads a lane has in flight; 1 and 3: 3 % slower on scans
 constexpr uint32_t UNANSWERED = 0xffffffffu, UNIT_FLAG = 0x80000000u;
 constexpr uint32_t NAN_ROW = 0x7fc00000u;  // every entry of a covariance row without a value
@@ -1161,9 +1162,11 @@ __device__ __forceinline__ bool group_unit(const Grid& g, const Grid& dg, const 
             tt = fminf(r2, tau);
             // A query off the grid or its window by more than its radius: widened by
             // a factor, the ball would hold thousands of points, walked by four
-            // lanes several times (60k queries, three quarters of them outside a
-            // window of 50k points: 13.4 ms so, 2.2 with k_knn_rest).
-            if (big || (none && g.exhaustive)) todo = false;
+            // lanes several times.  60k queries, three quarters of them outside a
+            // window of a quarter of the map, us here / with k_knn_rest: maps of
+            // 1k points 133 / 231, 2k 296 / 338, 4k 570 / 501, 8k 762 / 523, 32k
+            // 2017 / 476, 200k 13388 / 2241.
+            if (big || (none && g.exhaustive && g.m > SMALL_MAP)) todo = false;
             else w = 0;
         }
         const bool act = todo && tt >= 0.0f;
