@@ -51,67 +51,71 @@ __device__ __forceinline__ float box_eta(const Grid& g, float px, float py, floa
     return 0x1p-20f * (g.coord_scale + pm + (float)cm * g.h);
 }
 
-// Exact nearest map point of p among those with d2 <= max_d2: its position
-// in pts (or -1) and its d2.  A box of half-width r is searched for points
-// with d2 <= T = min(tau, max_d2); every point outside the box has d2 >
-// tau, so a hit is the global nearest, and no hit with tau >= max_d2 means
-// nothing lies within max_d2.  Otherwise r doubles.  When a box has more than
-// max_box_cells cells, the doubling starts once more, from r1 < r (so the wider
-// start, chosen for speed, costs no reach); after that such a box ends in a
-// linear scan of the whole map (exhaustive) or in `limited` with no pair.
-__device__ int nearest_within(const Grid& g, float px, float py, float pz, float max_d2, float r, float r1,
-                              float& bd2, bool& limited) {
-    // nothing beyond max_dist can pair: a box of this half-width (max_dist and the
-    // margins of certified_tau) settles the point
-    const float pm = fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz)));
-    const float r_max = sqrtf(max_d2) * (1.0f + 0x1p-12f) + 0x1p-18f * (g.coord_scale + pm);
-    r = fminf(r, r_max);
-    float seen = 0.0f;  // no point within it
-    for (int attempt = 0; attempt < 96; ++attempt) {
-        const int ulx = cell_of(__fsub_rn(px, r), g.ox, g.inv_h);
-        const int uhx = cell_of(__fadd_rn(px, r), g.ox, g.inv_h);
-        const int uly = cell_of(__fsub_rn(py, r), g.oy, g.inv_h);
-        const int uhy = cell_of(__fadd_rn(py, r), g.oy, g.inv_h);
-        const int ulz = cell_of(__fsub_rn(pz, r), g.oz, g.inv_h);
-        const int uhz = cell_of(__fadd_rn(pz, r), g.oz, g.inv_h);
-        const float tau = certified_tau(g, px, py, pz, ulx, uhx, uly, uhy, ulz, uhz);
-        const int lx = max(ulx, g.wlx), hx = min(uhx, g.whx);
-        const int ly = max(uly, g.wly), hy = min(uhy, g.why);
-        const int lz = max(ulz, g.wlz), hz = min(uhz, g.whz);
-        const int64_t ncl = (int64_t)max(hx - lx + 1, 0) * max(hy - ly + 1, 0) * max(hz - lz + 1, 0);
-        if (ncl > (int64_t)g.max_box_cells) {
-            if (!(r1 > 0.0f)) break;
-            while (r1 <= seen) r1 *= 2.0f;
-            r = r1;
-            r1 = 0.0f;
-            continue;
-        }
-        if (tau >= 0.0f) {
-            const float T = fminf(tau, max_d2);
-            u64 best = EMPTY_KEY;
-            uint32_t bpos = 0u;
-            if (ncl > 0) {
-                const float eta = box_eta(g, px, py, pz, ulx, uhx, uly, uhy, ulz, uhz);
-                auto visit = [&](uint32_t pos, const float4 q) {
-                    const float d = sqdist_pinned(px, py, pz, q.x, q.y, q.z);
-                    const u64 key = ((u64)__float_as_uint(d) << 32) | (u64)__float_as_uint(q.w);
-                    if (d <= T && key < best) {
-                        best = key;
-                        bpos = pos;
-                    }
-                };
-                if (g.dstart) for_rows(g, px, py, pz, lx, hx, ly, hy, lz, hz, eta, T, visit);
-                else for_box_points(g, px, py, pz, lx, hx, ly, hy, lz, hz, eta, T, visit);
+// One box of half-width r around p: 1 when it holds the exact nearest map point
+// within max_d2 (its position in pts and d2), 0 when nothing lies within max_d2,
+// -1 when neither is certain yet, -2 when it has more than max_box_cells cells.
+// It is searched for points with d2 <= T = min(tau, max_d2); every point outside
+// the box has d2 > tau, so a hit is the global nearest, and no hit with tau >=
+// max_d2 means nothing lies within max_d2.
+__device__ __forceinline__ int nearest_in_box(const Grid& g, float px, float py, float pz, float max_d2, float r,
+                                              int& pos, float& bd2) {
+    const int ulx = cell_of(__fsub_rn(px, r), g.ox, g.inv_h);
+    const int uhx = cell_of(__fadd_rn(px, r), g.ox, g.inv_h);
+    const int uly = cell_of(__fsub_rn(py, r), g.oy, g.inv_h);
+    const int uhy = cell_of(__fadd_rn(py, r), g.oy, g.inv_h);
+    const int ulz = cell_of(__fsub_rn(pz, r), g.oz, g.inv_h);
+    const int uhz = cell_of(__fadd_rn(pz, r), g.oz, g.inv_h);
+    const float tau = certified_tau(g, px, py, pz, ulx, uhx, uly, uhy, ulz, uhz);
+    const int lx = max(ulx, g.wlx), hx = min(uhx, g.whx);
+    const int ly = max(uly, g.wly), hy = min(uhy, g.why);
+    const int lz = max(ulz, g.wlz), hz = min(uhz, g.whz);
+    const int64_t ncl = (int64_t)max(hx - lx + 1, 0) * max(hy - ly + 1, 0) * max(hz - lz + 1, 0);
+    if (ncl > (int64_t)g.max_box_cells) return -2;
+    if (!(tau >= 0.0f)) return -1;
+    const float T = fminf(tau, max_d2);
+    u64 best = EMPTY_KEY;
+    uint32_t bpos = 0u;
+    if (ncl > 0) {
+        const float eta = box_eta(g, px, py, pz, ulx, uhx, uly, uhy, ulz, uhz);
+        auto visit = [&](uint32_t at, const float4 q) {
+            const float d = sqdist_pinned(px, py, pz, q.x, q.y, q.z);
+            const u64 key = ((u64)__float_as_uint(d) << 32) | (u64)__float_as_uint(q.w);
+            if (d <= T && key < best) {
+                best = key;
+                bpos = at;
             }
-            if (best != EMPTY_KEY) {
-                bd2 = __uint_as_float((uint32_t)(best >> 32));
-                return (int)bpos;
-            }
-            if (tau >= max_d2) return -1;
-            seen = r;
-        }
-        r = r < r_max ? fminf(r * 2.0f, r_max) : fminf(fmaxf(r, 0x1p-10f * g.h) * 2.0f, 1e30f);
+        };
+        if (g.dstart) for_rows(g, px, py, pz, lx, hx, ly, hy, lz, hz, eta, T, visit);
+        else for_box_points(g, px, py, pz, lx, hx, ly, hy, lz, hz, eta, T, visit);
     }
+    if (best != EMPTY_KEY) {
+        bd2 = __uint_as_float((uint32_t)(best >> 32));
+        pos = (int)bpos;
+        return 1;
+    }
+    return tau >= max_d2 ? 0 : -1;
+}
+
+// The search of a point whose boxes grew past max_box_cells: the doubling once
+// more, from r1 (so the wider start, chosen for speed, costs no reach) and past
+// `seen`, within which nothing lies; then a linear scan of the whole map
+// (exhaustive), or `limited` and no pair.  Out of line, with its lanes together:
+// in the pairing loop it slowed every other point (calls of 1k to 100k points
+// around 40 tight clusters, max_dist 0.1 m: 331-717 us before the second doubling,
+// 411-869 with it in the loop, 313-702 so; max_dist 1 m, most points scanning the
+// map: 22, 28, 18 ms for 20k).
+__device__ __noinline__ int nearest_past_limit(const Grid& g, float px, float py, float pz, float max_d2, float r1,
+                                               float seen, float& bd2, bool& limited) {
+    const unsigned together = __activemask();  // they scan the map side by side, not in turn
+    float r = r1;
+    while (r <= seen) r *= 2.0f;
+    int st = -1, pos = -1;
+    for (int attempt = 0; attempt < 48 && st == -1; ++attempt) {
+        st = nearest_in_box(g, px, py, pz, max_d2, r, pos, bd2);
+        r = fminf(r * 2.0f, 1e30f);
+    }
+    __syncwarp(together);
+    if (st >= 0) return pos;
     if (!g.exhaustive) {
         limited = true;
         return -1;
@@ -132,6 +136,24 @@ __device__ int nearest_within(const Grid& g, float px, float py, float pz, float
     if (best == EMPTY_KEY) return -1;
     bd2 = __uint_as_float((uint32_t)(best >> 32));
     return (int)bpos;
+}
+
+// Exact nearest map point of p among those with d2 <= max_d2: its position
+// in pts (or -1) and its d2, from boxes of half-width r, 2 r, ...
+__device__ __forceinline__ int nearest_within(const Grid& g, float px, float py, float pz, float max_d2, float r,
+                                              float r1, float& bd2, bool& limited) {
+    const unsigned together = __activemask();
+    float seen = 0.0f;
+    int st = -1, pos = -1;
+    for (int attempt = 0; attempt < 48; ++attempt) {
+        st = nearest_in_box(g, px, py, pz, max_d2, r, pos, bd2);
+        if (st != -1) break;
+        seen = r;
+        r = fminf(r * 2.0f, 1e30f);
+    }
+    __syncwarp(together);
+    if (st < 0) pos = nearest_past_limit(g, px, py, pz, max_d2, r1, seen, bd2, limited);
+    return pos;
 }
 
 // One pair's 29 terms in binary32 (all zero when S is not positive
@@ -211,7 +233,7 @@ __device__ __forceinline__ bool pair_terms(const float* R, float px, float py, f
 }
 
 __global__ void __launch_bounds__(GICP_THREADS) k_gicp_linearize(
-    Grid g, Grid dg, int has_delta, float2 r0d, const float* __restrict__ map_cov, const float* __restrict__ src,
+    const __grid_constant__ Grid g, const __grid_constant__ Grid dg, int has_delta, float2 r0d, const float* __restrict__ map_cov, const float* __restrict__ src,
     int64_t n, const float* __restrict__ src_cov, const float* __restrict__ pose, float max_d2, float2 r0,
     double* __restrict__ out, int32_t* __restrict__ corr, unsigned char* __restrict__ work) {
     __shared__ double red[GICP_THREADS / 32][GICP_STRIDE];
